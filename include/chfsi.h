@@ -24,9 +24,6 @@
  *
  * Environment variables (read once per process; none is needed for normal use)
  *   CHFSI_OZ_KERNEL=mma            digit products on the mma.sync kernel instead of tcgen05
- *   CHFSI_OZ_GROUPS=0              one slice pair per stage in the tcgen05 kernel (default:
- *                                  slice groups sharing one A tile, blocks <= 96 columns)
- *   CHFSI_OZ_GROUP_MIN_STAGES=k    smallest TMA ring a slice group may leave (default 4)
  *   CHFSI_SLICE_MARGIN_BITS=b      safety margin of the filter's per-loop slice count
  *                                  (default 6 bits)
  */

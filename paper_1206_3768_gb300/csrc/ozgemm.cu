@@ -101,6 +101,15 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
   lo += err;
 }
 
+// the same for a sc, sc a power of two (so that a sc is exact)
+__device__ __forceinline__ void two_sum_scaled(float& hi, float& lo, float a, float sc) {
+  const float s = fmaf(a, sc, hi);
+  const float bp = s - hi;
+  const float err = (hi - (s - bp)) + fmaf(a, sc, -bp);
+  hi = s;
+  lo += err;
+}
+
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const OzParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* sA = smem;                                    // stages x 128 x 64 bf16
@@ -260,71 +269,81 @@ __global__ void oz_epilogue_kernel(const double* part, int splits, int Mp, int N
 
 
 // ============================================================================ tcgen05 path
-// The same digit products on the 5th-generation tensor cores: TMA (128-byte swizzle) stages
-// a 128 x 64 bf16 tile of A and an (up to) 160 x 64 tile of B in shared memory, one elected
-// thread issues tcgen05.mma (kind::f16, bf16 inputs, FP32 accumulator in tensor memory, N up
-// to 160 so that a 130-column block is one tile and a 320-column block two), and sixteen
-// drain warps fold each exact 960-term chunk into double-float sums.  Tensor memory (512
-// columns): two sets of accumulators used alternately (one fills while the other drains) and
-// the high words of the sums after them; the low words live in the drain threads' registers.
-// Slice groups: the pairs are issued in groups (s, t0 .. t0 + g - 1) that share the A slice
-// s.  One stage holds one A tile and the B tiles of the whole group (consecutive slices of B
-// are consecutive rows of its buffer, so one TMA box of g x Np rows), and the MMA thread
-// issues the group's products into g accumulators.  The A stream then carries one tile per
-// group instead of one per pair.  g = 1 for blocks wider than 96 columns (two 160-column
-// accumulators at columns 0 and 160, high words at 320); narrower blocks take g up to 7 as
-// tensor memory allows: 2 g accumulators of the block's width (rounded up to 32 columns)
-// plus the high words.
-// Clusters: the CTAs of consecutive row tiles (2 or 4) form a cluster and share every B
-// tile: each CTA loads its share of the B box and multicasts it to the cluster, and the MMAs
-// of every CTA release a stage to all of them (the empty barriers count one arrival per
-// CTA), which divides the B stream from L2 by the cluster size.
-// Warp 0 issues TMA loads, warp 1 issues MMAs, warps 2..17 drain: four warps per group of 32
-// tensor-memory lanes; warp h of a lane group owns the 8-column blocks h, h + 4, ... of the
-// tile, so that narrow blocks still spread over all four.  18 warps allow 112 registers per
-// thread.  Every wait on an mbarrier is bounded; a wait that runs out sets DEV_TIMEOUT and the
-// CTA unwinds (waiting, again bounded, for its own copies and MMAs) before freeing tensor
-// memory.
-constexpr int TC_BM = 128, TC_BN = 160, TC_BK = 64;
-constexpr int TC_DWQ = 3;                                  // drain warps per 32-lane quarter
+// The same digit products on the 5th-generation tensor cores (tcgen05.mma, bf16 inputs, FP32
+// accumulators in tensor memory, operands staged by TMA).
+//
+// What bounds it: the tensor pipe needs 2 bytes of operand per 128 flops and tile row, and the
+// path from L2 into an SM carries about 30 to 40 bytes a clock.  A kernel that brings in one A
+// and one B tile for every slice pair (128 x 160 tile: 36 KB for 320 clocks of tensor work)
+// is therefore held at 28 % of the tensor rate.  Here a K-block of 64 brings in every slice of
+// both operands ONCE (S x 16 KB of A, S x 8 KB of B for a 64-column tile) and all S (S + 1) / 2
+// pairs (s, t) are issued from shared memory: 168 KB for 3584 clocks at S = 7, a third of the
+// bytes per flop.  Pairs of one level s + t carry the same scale 2^{-7 (s + t)} and add into
+// one accumulator, so S levels x 64 columns fit the 512 columns of tensor memory; the A slice s
+// meets the slices t = 1.. of B in ONE instruction of N = (number of levels) x w columns
+// (consecutive slices of B are consecutive rows of the stage, consecutive levels consecutive
+// accumulator columns), which also reads the A tile from shared memory once for several pairs.
+// Exactness: |digit 1| <= 129 and the others <= 64, so level l adds at most 129^2 (l = 2) or
+// 2 129 64 + (l - 3) 64^2 per k; a chunk of tc_chunk_kb(S) K-blocks keeps every level below
+// 2^24 and each chunk is exact in the FP32 accumulators.  Sixteen drain warps then add the
+// levels into double-float sums (hi, lo) held in their registers.
+// Regions: levels are split into regions of at most 256 accumulator columns (columns 0 and
+// 256).  With one region (S w <= 256) chunks alternate between the two halves of tensor
+// memory; with two, the first and the last K-block of a chunk issue region 0 (the larger
+// products) and then region 1, so that draining region 0 overlaps the last products of region
+// 1, and draining region 1 the first products of region 0 of the next chunk.
+// Measured against the one-pair-per-stage kernel (Gauss form, 7 slices, one product): n = 9300,
+// m = 320 6.1 -> 2.6 ms, 1.76 PFLOP/s of slice-pair flops at the card's power cap (2010 to 2070
+// MHz, 1360 W); n = 5957, m = 37 0.82 -> 0.25 ms; with 5 slices n = 2600, m = 130 and fewer
+// columns 0.15 -> 0.07 ms.
+// Warp 0 issues TMA loads (a ring of A tiles and a ring of B stages), warp 1 issues MMAs, warps
+// 2..17 drain: four warps per group of 32 tensor-memory lanes, warp h of a group owns the
+// 8-column blocks h and h + 4 of the tile.  Every wait on an mbarrier is bounded; a wait that
+// runs out sets DEV_TIMEOUT and the CTA unwinds (waiting, again bounded, for its own copies
+// and MMAs) before freeing tensor memory.
+constexpr int TC_BM = 128, TC_BK = 64;
+constexpr int TC_W = 64;                                   // widest column tile
+constexpr int TC_REGION = 256;                             // accumulator columns of a region
+constexpr int TC_DWQ = 4;                                  // drain warps per 32-lane quarter
 constexpr int TC_THREADS = 64 + 32 * 4 * TC_DWQ;           // producer, MMA issuer, drain warps
-// The ring holds as many stages as fit: 6 for a 144-row B box, up to TC_MAX_STAGES for narrow
-// blocks, whose smaller B boxes leave room for more of the (dominant) A stream in flight.
-constexpr int TC_MAX_STAGES = 12;
-constexpr int TC_SMEM_BUDGET = 227 * 1024 - 1024 - 512;  // dynamic shared memory for the ring
-constexpr int TC_DRAIN_THREADS = TC_THREADS - 64;
-constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;       // 16 KB per stage
-constexpr int TC_ACC1 = 160, TC_HI = 320;           // tensor-memory columns for groups of one
-constexpr int TC_LO = 480;                         // low words of tile columns 128..159
-constexpr int TC_GROUP_MAX_N = 96;                  // widest block issued in groups of g > 1
-constexpr int TC_GROUP_MAX = 7;
-static_assert((16 * TC_BK * 2) % 1024 == 0, "B stages (16-row multiples) stay 1024-byte aligned");
-static_assert(TC_HI + TC_BN <= TC_LO && TC_LO + (TC_BN - 128) <= 512 && TC_ACC1 + TC_BN <= TC_HI,
-              "tensor-memory layout");
+constexpr int TC_MAX_A = 12, TC_MAX_B = 4;                 // ring depths
+constexpr int TC_SMEM_BUDGET = 227 * 1024 - 1024 - 512;    // dynamic shared memory for the rings
+constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;              // 16 KB per A tile
+// Levels from this one on (s + t >= 7) go straight into the low word: a chunk of level 7 is about
+// 2^-33 of the operands' scales, so its rounding there is 2^-24 of that, below the rounding of
+// the low word itself (2^-48 of a sum near the scales) and the dropped pairs of 8 slices (2^-58
+// per term).  One instruction instead of seven per value.  From level 6 on it would cost
+// accuracy (reduction of n = 4096 with 8 slices: 3.4e-14 against 6.3e-15).
+constexpr int TC_LOW_LEVEL = 7;
+static_assert(8 * TC_W <= 512 && TC_W * (TC_REGION / TC_W) == TC_REGION && TC_W % 16 == 0 &&
+                  8 <= 2 * (TC_REGION / TC_W),
+              "eight levels fit two regions");
 constexpr long kMbarSpinLimit = 1L << 26;
+
+// K-blocks of 64 per exact chunk: the largest count that keeps the largest level below 2^24.
+constexpr int tc_chunk_kb(int S) {
+  const int top = 2 * 129 * 64 + (S - 2) * 64 * 64;  // level S + 1 (S >= 2)
+  const int per_k = S >= 3 && top > 129 * 129 ? top : 129 * 129;
+  return (1 << 24) / (per_k * TC_BK);
+}
+static_assert(tc_chunk_kb(1) == 15 && tc_chunk_kb(2) == 15 && tc_chunk_kb(7) == 7 && tc_chunk_kb(8) == 6,
+              "exact chunks");
 
 struct TcParams {
   int a_lower, c_lower;                      // as in OzParams
   int b_tri;                                 // op(B) (complex) zero for k > j (1) or k < j (2)
-  int nkb, tiles_m, splits, Mp, Np, n_real;  // n_real: columns of B^ that hold data
-  int b_box_rows;                            // rows of the B box (<= TC_BN, multiple of 16)
-  int stages;                                // TMA ring depth (<= TC_MAX_STAGES)
-  int pair_split;                            // splits partition the slice groups (else k-blocks)
-  int group;                                 // g: largest group (B box = g x Np rows when g > 1)
-  int acc_stride;                            // tensor-memory columns between accumulators
-  int ngroups;
-  unsigned char gs[OZ_MAX_PAIRS], gt[OZ_MAX_PAIRS], gc[OZ_MAX_PAIRS];  // group: s, first t, size
+  int S;                                     // slices (levels)
+  int w;                                     // columns per tile (multiple of 16, <= TC_W)
+  int nkb, tiles_m, tiles_n, raster, splits, Mp, Np;
+  int na, nb;                                // ring depths: A tiles, B stages
+  int chunk_kb;                              // K-blocks per exact chunk
+  int a_zslices, b_zslices;                  // slices between the products of the Gauss form
   double* part;
   int* status;
   long long spin_limit;                      // polls before a first-level wait gives up
-  int cl;                                    // CTAs per cluster along M sharing the B tiles (1, 2, 4)
-  int tiles_m_pad;                           // tiles_m rounded up to a multiple of cl
-  int col_major_order;                       // 1: blockIdx.x runs over column tiles first (cl == 1)
   // Gauss form (nz = 3): blockIdx.z picks one of three real products whose operands follow
-  // each other in the slice buffers (a_zrows rows of A, b_zrows rows of B apart) and whose
-  // split partials follow each other in part (splits x Mp x Np entries apart)
-  int nz;
-  int a_zrows, b_zrows;
+  // each other in the slice buffers and whose split partials follow each other in part
+  // (splits x Mp x Np entries apart)
   int kfac;  // real k (and rows of A) per complex index: 2 in the embedding, 1 in the Gauss form
 };
 
@@ -335,7 +354,7 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes));
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar));
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -343,7 +362,8 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(bar), "r"(parity));
+      : "r"(bar), "r"(parity)
+      : "memory");
   return ok != 0;
 }
 // Bounded wait: false (with DEV_TIMEOUT set and the CTA's abort flag raised) if it ran out
@@ -365,31 +385,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return true;
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z,
                                             uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
       : "memory");
 }
-// The same copy delivered to every CTA of the cluster in `mask`, at the same shared-memory
-// offsets (destination and mbarrier) as this CTA's.
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                               uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1, {%2, %3}], [%4], %5;\n"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
-      : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_ctarank() {
+
+// True for one lane of a converged warp.  The producer and the MMA issuer run under this
+// election rather than under lane == 0: the tensor instructions take their operands from
+// uniform registers, and a branch the compiler knows to be uniform issues them at 39 clocks
+// each and a commit at about 100, against 53 and 250 (measured with N = 16).
+__device__ __forceinline__ bool elect_one() {
   uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
 }
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, 8-row groups 1024 B apart.
@@ -419,12 +430,6 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
                ::"r"(bar) : "memory");
 }
-// Arrive (once the issued MMAs complete) on the mbarrier at this offset in every CTA of mask.
-__device__ __forceinline__ void tc_commit_mc(uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
-      ::"r"(bar), "h"(mask) : "memory");
-}
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 }
@@ -437,21 +442,128 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
-               ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]));
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* v) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n"
-               ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]));
-}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
+
+// The MMA issuer's state: one elected thread walks the K-blocks of its CTA.
+struct IssueArgs {
+  uint32_t sA, sB, b_slice, b_stage;               // shared-memory addresses and sizes
+  uint32_t fullA, emptyA, fullB, emptyB, accf, acce;  // mbarriers
+  uint32_t tmem;
+  int w, NA, NB, kb_lo, kb_hi, chunk_kb;
+  volatile int* abort_flag;
+  int* status;
+  long long spin_limit;
+};
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                            int* status, long long limit) {
+  return mbar_wait(bar, parity, abort_flag, status, limit);
+}
+__device__ __forceinline__ bool issue_wait(uint32_t bar, uint32_t parity, const IssueArgs& a) {
+  return mbar_try(bar, parity) || mbar_wait_slow(bar, parity, a.abort_flag, a.status, a.spin_limit);
+}
+// Descriptors of one operand differ in their low word only (the start address).
+__device__ __forceinline__ uint64_t desc_from(uint32_t lo, uint32_t hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(d) : "r"(lo), "r"(hi));
+  return d;
+}
+
+// S slices, U levels per region.  A K-block is S waits, up to 2 S groups of four products and S
+// commits; the loops over slices and regions are unrolled because one thread issues all of it
+// and its address arithmetic, not the tensor pipe, set the pace of a rolled loop (n = 9300, m =
+// 320: 3.5 ms a product).
+template <int S, int U>
+__device__ __forceinline__ void issue_products(const IssueArgs& a) {
+  constexpr int NREG = S > U ? 2 : 1;
+  const uint32_t desc_hi = (uint32_t)(sw128_desc(0) >> 32), desc_lo = (uint32_t)sw128_desc(0);
+  const uint32_t idesc0 = idesc_bf16(TC_BM, 0), idesc_w = (uint32_t)(a.w >> 3) << 17;
+  const uint32_t b_slice16 = a.b_slice >> 4;
+  int chunk = 0, sa = 0, sb = 0;
+  uint32_t pa = 0, pb = 0;
+  for (int k0 = a.kb_lo; k0 < a.kb_hi; k0 += a.chunk_kb, ++chunk) {
+    const int k1 = min(a.kb_hi, k0 + a.chunk_kb);
+    for (int kb = k0; kb < k1; ++kb) {
+      if (!issue_wait(a.fullB + 8 * sb, pb, a)) return;
+      const uint32_t b_lo = desc_lo + ((a.sB + (uint32_t)sb * a.b_stage) >> 4);
+      const bool first = kb == k0, last = kb == k1 - 1;
+      // group of four products of slice s into region `reg`: levels max(l0, s) .. l1 - 1
+      auto group = [&](int s, int reg, uint32_t a_lo) -> bool {
+        const int l0 = reg * U, l1 = S < l0 + U ? S : l0 + U;
+        const int lb = l0 > s ? l0 : s;
+        const uint32_t r = NREG == 2 ? (uint32_t)reg : (uint32_t)(chunk & 1);
+        if (s == 0 && first) {
+          // the region is free once the drain has finished its previous use
+          const int use = NREG == 2 ? chunk : (chunk >> 1);
+          if (use >= 1 && !issue_wait(a.acce + 8 * r, (use - 1) & 1, a)) return false;
+          tc_fence_after();
+        }
+        const uint32_t idesc = idesc0 + (uint32_t)(l1 - lb) * idesc_w;
+        const uint32_t d = a.tmem + r * TC_REGION + (uint32_t)((lb - l0) * a.w);
+        const uint32_t bl = b_lo + (uint32_t)(lb - s) * b_slice16;
+        // the first product of a chunk (s = 0 reaches every level) overwrites the region
+        const uint32_t keep = (s == 0 && first) ? 0u : 1u;
+#pragma unroll
+        for (int kk = 0; kk < TC_BK / 16; ++kk)  // 16 k = 32 bytes = 2 descriptor units
+          tc_mma(d, desc_from(a_lo + 2 * kk, desc_hi), desc_from(bl + 2 * kk, desc_hi), idesc, kk ? 1u : keep);
+        return true;
+      };
+      int slot = sa;
+      uint32_t ph = pa;
+      auto next_slot = [&] {
+        if (++slot == a.NA) {
+          slot = 0;
+          ph ^= 1;
+        }
+      };
+      auto a_lo_of = [&](int sl) { return desc_lo + ((a.sA + (uint32_t)sl * TC_A_BYTES) >> 4); };
+      if (NREG == 2 && (first || last)) {
+        // the first and the last K-block of a chunk issue region 0 and then region 1 (see the
+        // header); the A tiles below U stay until their second use
+#pragma unroll
+        for (int s = 0; s < U; ++s) {
+          if (!issue_wait(a.fullA + 8 * slot, ph, a)) return;
+          tc_fence_after();
+          if (!group(s, 0, a_lo_of(slot))) return;
+          next_slot();
+        }
+        if (last) tc_commit(a.accf);
+        slot = sa;
+        ph = pa;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (s >= U) {
+            if (!issue_wait(a.fullA + 8 * slot, ph, a)) return;
+            tc_fence_after();
+          }
+          if (!group(s, 1, a_lo_of(slot))) return;
+          tc_commit(a.emptyA + 8 * slot);
+          next_slot();
+        }
+        if (last) tc_commit(a.accf + 8);
+      } else {
+        // the others slice by slice, which releases the A tiles earlier
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (!issue_wait(a.fullA + 8 * slot, ph, a)) return;
+          tc_fence_after();
+          const uint32_t al = a_lo_of(slot);
+          if (s < U && !group(s, 0, al)) return;
+          if (NREG == 2 && !group(s, 1, al)) return;
+          tc_commit(a.emptyA + 8 * slot);
+          next_slot();
+        }
+        if (NREG == 1 && last) tc_commit(a.accf + 8 * (chunk & 1));
+      }
+      tc_commit(a.emptyB + 8 * sb);
+      sa = slot;
+      pa = ph;
+      if (++sb == a.NB) {
+        sb = 0;
+        pb ^= 1;
+      }
+    }
+  }
+}
 
 __global__ void __launch_bounds__(TC_THREADS, 1)
     oz_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -459,72 +571,60 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   extern __shared__ unsigned char tc_smem_raw[];
   const uintptr_t base = (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023;
   unsigned char* sA = reinterpret_cast<unsigned char*>(base);
-  const int NS = p.stages, b_stage = p.b_box_rows * TC_BK * 2;  // B stage bytes: a multiple of 2048
-  unsigned char* sB = sA + NS * TC_A_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sB + NS * b_stage);
-  // bars: full[STAGES], empty[STAGES], accf[2], acce[2], done[1]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * NS + 5);
+  const int S = p.S, w = p.w, NA = p.na, NB = p.nb;
+  const uint32_t b_slice = (uint32_t)w * (TC_BK * 2), b_stage = (uint32_t)S * b_slice;  // multiples of 2048
+  unsigned char* sB = sA + NA * TC_A_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sB + NB * b_stage);
+  // bars: fullA[NA], emptyA[NA], fullB[NB], emptyB[NB], accf[2], acce[2], done[1]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * (NA + NB) + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // tile order: row tiles fastest, or (col_major_order) the column tiles of one row tile next
-  // to each other, so that they stream the same A panels at about the same time
-  const int tiles_n = (int)(gridDim.x / (unsigned)p.tiles_m_pad);
-  const int tm = p.col_major_order ? (int)blockIdx.x / tiles_n : (int)blockIdx.x % p.tiles_m_pad;
-  const int tn = p.col_major_order ? (int)blockIdx.x % tiles_n : (int)blockIdx.x / p.tiles_m_pad;
-  const int m0 = tm * TC_BM, n0 = tn * TC_BN;
-  // Clusters of p.cl CTAs on consecutive row tiles share every B tile: each CTA loads 1/cl of
-  // the B box and multicasts it to the whole cluster, so all CTAs of a cluster must walk the
-  // same stages.  Their work is therefore decided by the cluster's last row tile (the widest
-  // k-range of a lower-triangular A, the last tile to reach the diagonal); the extra work is
-  // exact (zero blocks of A) or unused (tiles above the diagonal, rows past Mp).
-  const int crank = p.cl > 1 ? (int)cluster_ctarank() : 0;
-  const int m0_last = (tm - crank + p.cl - 1) * TC_BM;
-  const uint16_t cmask = (uint16_t)((1u << p.cl) - 1u);
-  if (p.c_lower && n0 > (m0_last + TC_BM - 1) / p.kfac) return;  // above the diagonal: not needed
-  // k-blocks of this CTA: split y takes [y per, (y + 1) per) of the tile's nonzero k-blocks.
-  // The work is ordered panel-major: for each panel of at most OZ_CHUNK_KB k-blocks, every
-  // slice pair in turn (one exact chunk each), so consecutive chunks reuse the same panel of
-  // an A slice from L2 while it is hot.
-  const int ncols = min(TC_BN, ((p.n_real - n0 + 15) / 16) * 16);  // MMA N for this tile
+  // Tile order: groups of p.raster column tiles; within a group the column tiles of a row tile
+  // are neighbours (they stream the same A slices at about the same time), row tiles follow.
+  // With a lower-triangular A the row tiles with the longest k-range start first.
+  int tm, tn;
+  {
+    const int per_group = p.tiles_m * p.raster;
+    const int g = (int)blockIdx.x / per_group, r = (int)blockIdx.x - g * per_group;
+    const int gw = min(p.raster, p.tiles_n - g * p.raster);
+    tm = r / gw;
+    tn = g * p.raster + (r - tm * gw);
+    if (p.a_lower) tm = p.tiles_m - 1 - tm;
+  }
+  const int m0 = tm * TC_BM, n0 = tn * w;
+  if (p.c_lower && n0 > (m0 + TC_BM - 1) / p.kfac) return;  // above the diagonal: not needed
   // nonzero k-blocks of the tile (k in real units, kfac per complex index): below
   // (m0 + 128) / 64 for a lower-triangular A (rows are in the same units); from kfac n0 / 64
-  // for a lower-triangular B (zero for k < j); below kfac (n0 + ncols) / 64 for an
+  // for a lower-triangular B (zero for k < j); below kfac (n0 + w) / 64 for an
   // upper-triangular B (zero for k > j)
-  int kb_first = 0, nkb = p.a_lower ? min(p.nkb, m0_last / TC_BK + TC_BM / TC_BK) : p.nkb;
+  int kb_first = 0, nkb = p.a_lower ? min(p.nkb, m0 / TC_BK + TC_BM / TC_BK) : p.nkb;
   if (p.b_tri == 2) kb_first = min(nkb, (p.kfac * n0) / TC_BK);
-  if (p.b_tri == 1) nkb = min(nkb, (p.kfac * (n0 + ncols) + TC_BK - 1) / TC_BK);
-  // split y takes either a range of k-blocks (all groups) or, for short K (one panel), a
-  // range of slice groups (all k-blocks)
-  int kb_lo = kb_first, kb_hi = nkb, pr_lo = 0, pr_hi = p.ngroups;
-  if (p.pair_split) {
-    const int pp = (p.ngroups + p.splits - 1) / p.splits;
-    pr_lo = min(p.ngroups, (int)blockIdx.y * pp);
-    pr_hi = min(p.ngroups, pr_lo + pp);
-  } else {
-    const int per = (nkb - kb_first + p.splits - 1) / p.splits;
-    kb_lo = min(nkb, kb_first + (int)blockIdx.y * per);
-    kb_hi = min(nkb, kb_lo + per);
-  }
-  const int npr = pr_hi - pr_lo;
-  // tensor-memory columns: accumulator j of buffer b at (b g + j) acc_stride, high words after
-  const int G = p.group;
-  const uint32_t acc_stride = (uint32_t)p.acc_stride, hi_col = 2u * (uint32_t)G * acc_stride;
-  const uint32_t b_pair_bytes = (uint32_t)p.Np * TC_BK * 2;  // B tile of one slice in a group box
-  const int b_share = p.b_box_rows / p.cl;                   // B rows each CTA of a cluster loads
+  if (p.b_tri == 1) nkb = min(nkb, (p.kfac * (n0 + w) + TC_BK - 1) / TC_BK);
+  // split y takes the k-blocks [y per, (y + 1) per) of them
+  const int per = (nkb - kb_first + p.splits - 1) / p.splits;
+  const int kb_lo = min(nkb, kb_first + (int)blockIdx.y * per);
+  const int kb_hi = min(nkb, kb_lo + per);
+  const int U = min(S, TC_REGION / w);  // levels per region
+  const int nreg = S > U ? 2 : 1;
 
   const uint32_t sA_u = smem_u32(sA), sB_u = smem_u32(sB);
-  const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * NS;
-  const uint32_t accf0 = empty0 + 8 * NS, acce0 = accf0 + 16, done_bar = acce0 + 16;
+  const uint32_t fullA = smem_u32(bars), emptyA = fullA + 8 * NA;
+  const uint32_t fullB = emptyA + 8 * NA, emptyB = fullB + 8 * NB;
+  const uint32_t accf0 = emptyB + 8 * NB, acce0 = accf0 + 16, done_bar = acce0 + 16;
 
   if (tid == 0) {
-    for (int i = 0; i < NS; ++i) {
-      mbar_init(full0 + 8 * i, 1);
-      mbar_init(empty0 + 8 * i, p.cl);  // released by the MMAs of every CTA of the cluster
+    for (int i = 0; i < NA; ++i) {
+      mbar_init(fullA + 8 * i, 1);
+      mbar_init(emptyA + 8 * i, 1);
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(accf0 + 8 * b, 1);
-      mbar_init(acce0 + 8 * b, TC_DRAIN_THREADS);
+    for (int i = 0; i < NB; ++i) {
+      mbar_init(fullB + 8 * i, 1);
+      mbar_init(emptyB + 8 * i, 1);
+    }
+    for (int r = 0; r < 2; ++r) {
+      mbar_init(accf0 + 8 * r, 1);
+      mbar_init(acce0 + 8 * r, 4 * TC_DWQ);  // one arrival per drain warp
     }
     mbar_init(done_bar, 1);
     *abort_flag = 0;
@@ -535,103 +635,84 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         smem_u32(tmem_slot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
+  tc_fence_before();
   __syncthreads();
-  // every CTA of the cluster has initialised its barriers before any copy or commit reaches them
-  if (p.cl > 1) cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      // ring position kept incrementally (no division on this single-thread issue path)
-      int i = 0, stage = 0;
-      uint32_t phase = 0;
+    if (elect_one()) {
+      // ring positions kept incrementally (no division on this single-thread issue path)
+      int ia = 0, ib = 0, sa = 0, sb = 0;
+      uint32_t pa = 0, pb = 0;
       bool stop = false;
-      for (int k0 = kb_lo; k0 < kb_hi && !stop; k0 += OZ_CHUNK_KB) {
-        const int k1 = min(kb_hi, k0 + OZ_CHUNK_KB);
-        for (int pr = pr_lo; pr < pr_hi && !stop; ++pr) {
-          const int arow = (int)blockIdx.z * p.a_zrows + p.gs[pr] * p.Mp + m0;
-          const int brow = (int)blockIdx.z * p.b_zrows + p.gt[pr] * p.Np + n0;
-          for (int kb = k0; kb < k1; ++kb, ++i) {
-            const uint32_t fb = full0 + 8 * stage;
-            if (i >= NS && !mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, p.spin_limit)) {
-              stop = true;
-              break;
-            }
-            mbar_expect_tx(fb, TC_A_BYTES + b_stage);
-            tma_load_2d(sA_u + stage * TC_A_BYTES, &tmA, kb * TC_BK, arow, fb);
-            if (p.cl > 1)  // this CTA's share of the B box, to every CTA of the cluster
-              tma_load_2d_mc(sB_u + stage * b_stage + (uint32_t)(crank * b_share) * (TC_BK * 2), &tmB,
-                             kb * TC_BK, brow + crank * b_share, fb, cmask);
-            else
-              tma_load_2d(sB_u + stage * b_stage, &tmB, kb * TC_BK, brow, fb);
-            if (++stage == NS) {
-              stage = 0;
-              phase ^= 1;
-            }
+      const int az = (int)blockIdx.z * p.a_zslices, bz = (int)blockIdx.z * p.b_zslices;
+      for (int kb = kb_lo; kb < kb_hi && !stop; ++kb) {
+        if (ib >= NB && !mbar_wait(emptyB + 8 * sb, pb ^ 1, abort_flag, p.status, p.spin_limit)) break;
+        mbar_expect_tx(fullB + 8 * sb, b_stage);
+        tma_load_3d(sB_u + (uint32_t)sb * b_stage, &tmB, kb * TC_BK, n0, bz, fullB + 8 * sb);
+        ++ib;
+        if (++sb == NB) {
+          sb = 0;
+          pb ^= 1;
+        }
+        for (int s = 0; s < S; ++s) {
+          if (ia >= NA && !mbar_wait(emptyA + 8 * sa, pa ^ 1, abort_flag, p.status, p.spin_limit)) {
+            stop = true;
+            break;
+          }
+          mbar_expect_tx(fullA + 8 * sa, TC_A_BYTES);
+          tma_load_3d(sA_u + (uint32_t)sa * TC_A_BYTES, &tmA, kb * TC_BK, m0, az + s, fullA + 8 * sa);
+          ++ia;
+          if (++sa == NA) {
+            sa = 0;
+            pa ^= 1;
           }
         }
       }
-      // on abort: let the copies already issued (stages i - STAGES .. i - 1) land before the
-      // CTA can exit
+      // on abort: let the copies already issued (the last NA tiles and NB stages) land before
+      // the CTA can exit
       if (*abort_flag) {
-        for (int j = max(0, i - NS); j < i; ++j) {
+        for (int j = max(0, ia - NA); j < ia; ++j) {
           long it = 0;
-          while (!mbar_try(full0 + 8 * (j % NS), (j / NS) & 1) && ++it < kMbarSpinLimit) {}
+          while (!mbar_try(fullA + 8 * (j % NA), (j / NA) & 1) && ++it < kMbarSpinLimit) {}
         }
-      } else if (p.cl > 1) {
-        // the B shares this CTA sent to the cluster: every CTA has consumed them (so they have
-        // landed) before this CTA may exit
-        for (int j = max(0, i - NS); j < i; ++j) {
+        for (int j = max(0, ib - NB); j < ib; ++j) {
           long it = 0;
-          while (!mbar_try(empty0 + 8 * (j % NS), (j / NS) & 1) && ++it < kMbarSpinLimit) {}
+          while (!mbar_try(fullB + 8 * (j % NB), (j / NB) & 1) && ++it < kMbarSpinLimit) {}
         }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(TC_BM, ncols);
-      int chunk = 0, stage = 0;
-      uint32_t phase = 0;
-      bool stop = false;
-      for (int k0 = kb_lo; k0 < kb_hi && !stop; k0 += OZ_CHUNK_KB) {
-        const int k1 = min(kb_hi, k0 + OZ_CHUNK_KB);
-        for (int pr = pr_lo; pr < pr_hi && !stop; ++pr, ++chunk) {
-          // accumulator chunk & 1 is free once the drain has finished chunk - 2
-          if (chunk >= 2 && !mbar_wait(acce0 + 8 * (chunk & 1), ((chunk >> 1) - 1) & 1, abort_flag, p.status,
-                                     p.spin_limit)) {
-            stop = true;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)(chunk & 1) * (uint32_t)G * acc_stride;
-          const int gc = p.gc[pr];
-          for (int kb = k0; kb < k1; ++kb) {
-            if (!mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, p.spin_limit)) {
-              stop = true;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t a_s = sA_u + stage * TC_A_BYTES, b_s = sB_u + stage * b_stage;
-            // pair j of the group: B tile j of the box into accumulator j
-            for (int j = 0; j < gc; ++j) {
-#pragma unroll
-              for (int kk = 0; kk < TC_BK / 16; ++kk)
-                tc_mma(d + (uint32_t)j * acc_stride, sw128_desc(a_s + kk * 32),
-                       sw128_desc(b_s + (uint32_t)j * b_pair_bytes + kk * 32), idesc,
-                       (kb == k0 && kk == 0) ? 0u : 1u);
-            }
-            if (p.cl > 1) tc_commit_mc(empty0 + 8 * stage, cmask);
-            else tc_commit(empty0 + 8 * stage);
-            if (kb == k1 - 1) tc_commit(accf0 + 8 * (chunk & 1));
-            if (++stage == NS) {
-              stage = 0;
-              phase ^= 1;
-            }
-          }
-        }
+    if (elect_one()) {
+      IssueArgs ia;
+      ia.sA = sA_u; ia.sB = sB_u; ia.b_slice = b_slice; ia.b_stage = b_stage;
+      ia.fullA = fullA; ia.emptyA = emptyA; ia.fullB = fullB; ia.emptyB = emptyB;
+      ia.accf = accf0; ia.acce = acce0;
+      ia.tmem = tmem;
+      ia.w = w; ia.NA = NA; ia.NB = NB; ia.kb_lo = kb_lo; ia.kb_hi = kb_hi; ia.chunk_kb = p.chunk_kb;
+      ia.abort_flag = abort_flag; ia.status = p.status; ia.spin_limit = p.spin_limit;
+      // one unrolled loop per (slices, levels per region); U = 4 (w = 64) and 5 (w = 48) leave two
+      // regions for more slices than that, all other widths one
+      switch (nreg == 2 ? 16 * U + S : S) {
+        case 1: issue_products<1, 1>(ia); break;
+        case 2: issue_products<2, 2>(ia); break;
+        case 3: issue_products<3, 3>(ia); break;
+        case 4: issue_products<4, 4>(ia); break;
+        case 5: issue_products<5, 5>(ia); break;
+        case 6: issue_products<6, 6>(ia); break;
+        case 7: issue_products<7, 7>(ia); break;
+        case 8: issue_products<8, 8>(ia); break;
+        case 16 * 4 + 5: issue_products<5, 4>(ia); break;
+        case 16 * 4 + 6: issue_products<6, 4>(ia); break;
+        case 16 * 4 + 7: issue_products<7, 4>(ia); break;
+        case 16 * 4 + 8: issue_products<8, 4>(ia); break;
+        case 16 * 5 + 6: issue_products<6, 5>(ia); break;
+        case 16 * 5 + 7: issue_products<7, 5>(ia); break;
+        case 16 * 5 + 8: issue_products<8, 5>(ia); break;
+        default: break;  // no other (S, w) is launched
       }
       // all MMAs issued by this thread are complete once done_bar fires
       tc_commit(done_bar);
@@ -639,136 +720,71 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       while (!mbar_try(done_bar, 0) && ++it < kMbarSpinLimit) {}
     }
   } else {
-    // ------------------------------------------------------------ drain warps (2..13)
-    // Thread (quarter, lane) of warp h (0..2 within its lane group) owns row 32 * quarter +
-    // lane of the tile and the 8-column blocks h + 3 i: the high words of its sums sit in
-    // tensor memory, the low words of columns 0..127 in lo[] (registers; the block loops below
-    // are unrolled so that every index into lo[] is a constant) and those of columns 128..159
-    // in the last 32 tensor-memory columns (blocks 16..19 are only used with groups of one,
-    // whose high words end at column 480).  Tensor memory is moved in blocks of 8 columns to
-    // keep the live registers within the 128 that 14 warps allow.
-    const int quarter = warp & 3;  // tensor-memory lanes 32*quarter .. +31
-    constexpr int kRegCols = 128;                                       // columns with lo[] in registers
-    constexpr int kBlocks = (kRegCols / 8 + TC_DWQ - 1) / TC_DWQ;       // register blocks per warp
-    constexpr int kTmBlocks = ((TC_BN - kRegCols) / 8 + TC_DWQ - 1) / TC_DWQ;  // tensor-memory blocks
-    const int h = (warp - 2) >> 2;
+    // ------------------------------------------------------------ drain warps (2..17)
+    // Thread (quarter, lane) of warp h (0..3 of its lane group) owns row 32 * quarter + lane of
+    // the tile and the 8-column blocks h and h + 4.
+    const int quarter = warp & 3, h = (warp - 2) >> 2, nblk = w >> 3;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    const int reg_cols = min(ncols, kRegCols);
-    float lo[kBlocks * 8];
-    {
-      uint32_t zero[8];
+    float hi[2][8], lo[2][8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) zero[j] = 0u;
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int c = 0; c < kBlocks; ++c) {
-        // only the tile's columns: with groups the high words end at the last allocated column
-        const int col = 8 * (TC_DWQ * c + h);
-        if (col < reg_cols) tmem_st8(lane_base + hi_col + col, zero);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) lo[c * 8 + j] = 0.f;
-      }
-#pragma unroll
-      for (int t = 0; t < kTmBlocks; ++t) {
-        const int col = kRegCols + 8 * (TC_DWQ * t + h);
-        if (col < ncols) {
-          tmem_st8(lane_base + hi_col + col, zero);
-          tmem_st8(lane_base + TC_LO + (col - kRegCols), zero);
-        }
-      }
-      tmem_wait_st();
-    }
-    int chunk = 0;
+      for (int q = 0; q < 8; ++q) hi[i][q] = lo[i][q] = 0.f;
+    const int nchunks = kb_hi > kb_lo ? (kb_hi - kb_lo + p.chunk_kb - 1) / p.chunk_kb : 0;
     bool ok = true;
-    const int nchunks = (kb_hi > kb_lo && npr > 0) ? ((kb_hi - kb_lo + OZ_CHUNK_KB - 1) / OZ_CHUNK_KB) * npr : 0;
-    for (; chunk < nchunks && ok; ++chunk) {
-      const int b = chunk & 1;
-      if (!mbar_wait(accf0 + 8 * b, (chunk >> 1) & 1, abort_flag, p.status, p.spin_limit, true)) { ok = false; break; }
+    for (int use = 0; use < nchunks * nreg && ok; ++use) {
+      const int r = use & 1;  // regions alternate in both forms
+      if (!mbar_wait(accf0 + 8 * r, (use >> 1) & 1, abort_flag, p.status, p.spin_limit, true)) {
+        ok = false;
+        break;
+      }
       tc_fence_after();
-      const int pr = pr_lo + chunk % npr;
-      const int gc = p.gc[pr];
-      const float sc0 = ldexpf(1.0f, -OZ_BETA * (p.gs[pr] + p.gt[pr] + 2));
-      const uint32_t acc_base = lane_base + (uint32_t)b * (uint32_t)G * acc_stride;
+      const int l0 = (nreg == 2 && r) ? U : 0, nl = min(S - l0, U);
+      const uint32_t acc_base = lane_base + (uint32_t)(r * TC_REGION);
 #pragma unroll
-      for (int c = 0; c < kBlocks; ++c) {
-        const int col = 8 * (TC_DWQ * c + h);
-        if (col < reg_cols) {
-          uint32_t acc[8], hi[8];
-          tmem_ld8(lane_base + hi_col + col, hi);
-          float sc = sc0;
-          for (int j = 0; j < gc; ++j) {  // pair (s, t0 + j), scale 2^{-7 (s + t0 + j + 2)}
-            tmem_ld8(acc_base + (uint32_t)j * acc_stride + col, acc);
+      for (int i = 0; i < 2; ++i) {
+        const int blk = h + 4 * i;
+        if (blk < nblk) {
+          for (int l = 0; l < nl; l += 4) {
+            uint32_t acc[4][8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (l + q < nl) tmem_ld8(acc_base + (uint32_t)((l + q) * w + 8 * blk), acc[q]);
             tmem_wait_ld();
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              float hq = __uint_as_float(hi[q]);
-              two_sum_acc(hq, lo[c * 8 + q], __uint_as_float(acc[q]) * sc);
-              hi[q] = __float_as_uint(hq);
-            }
-            sc *= 0.0078125f;  // 2^-7
-          }
-          tmem_st8(lane_base + hi_col + col, hi);
-        }
-      }
+            for (int q = 0; q < 4; ++q)
+              if (l + q < nl) {
+                // level l0 + l + q (0-based) carries 2^{-7 (level + 2)}
+                const int level = l0 + l + q + 2;
+                const float sc = __int_as_float((127 - OZ_BETA * level) << 23);
+                if (level < TC_LOW_LEVEL) {
 #pragma unroll
-      for (int t = 0; t < kTmBlocks; ++t) {  // groups of one: a single pair per chunk
-        const int col = kRegCols + 8 * (TC_DWQ * t + h);
-        if (col < ncols) {
+                  for (int c = 0; c < 8; ++c) two_sum_scaled(hi[i][c], lo[i][c], __uint_as_float(acc[q][c]), sc);
+                } else {
 #pragma unroll
-          for (int half = 0; half < 8; half += 4) {  // four columns at a time (registers)
-            uint32_t acc[4], hi[4], lw[4];
-            tmem_ld4(lane_base + hi_col + col + half, hi);
-            tmem_ld4(lane_base + TC_LO + (col - kRegCols) + half, lw);
-            tmem_ld4(acc_base + col + half, acc);
-            tmem_wait_ld();
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float hq = __uint_as_float(hi[q]), lq = __uint_as_float(lw[q]);
-              two_sum_acc(hq, lq, __uint_as_float(acc[q]) * sc0);
-              hi[q] = __float_as_uint(hq);
-              lw[q] = __float_as_uint(lq);
-            }
-            tmem_st4(lane_base + hi_col + col + half, hi);
-            tmem_st4(lane_base + TC_LO + (col - kRegCols) + half, lw);
+                  for (int c = 0; c < 8; ++c) lo[i][c] = fmaf(__uint_as_float(acc[q][c]), sc, lo[i][c]);
+                }
+              }
           }
         }
       }
-      tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(acce0 + 8 * b);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce0 + 8 * r);
     }
-    if (ok && !*abort_flag && m0 < p.Mp) {
+    if (ok && !*abort_flag) {
       // partial sums of this split as (hi, lo) pairs: P[split][col * Mp + row]
       float2* P = reinterpret_cast<float2*>(p.part) +
                   ((int64_t)blockIdx.z * p.splits + blockIdx.y) * p.Mp * p.Np;
       const int row = m0 + quarter * 32 + lane;
 #pragma unroll
-      for (int c = 0; c < kBlocks; ++c) {
-        const int col0 = 8 * (TC_DWQ * c + h);
-        if (col0 < reg_cols) {
-          uint32_t hi[8];
-          tmem_ld8(lane_base + hi_col + col0, hi);
-          tmem_wait_ld();
+      for (int i = 0; i < 2; ++i) {
+        const int blk = h + 4 * i;
+        if (blk < nblk) {
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int col = n0 + col0 + q;
-            if (col < p.Np)
-              P[(int64_t)col * p.Mp + row] = make_float2(__uint_as_float(hi[q]), lo[c * 8 + q]);
-          }
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < kTmBlocks; ++t) {
-        const int col0 = kRegCols + 8 * (TC_DWQ * t + h);
-        if (col0 < ncols) {
-          uint32_t hi[8], lw[8];
-          tmem_ld8(lane_base + hi_col + col0, hi);
-          tmem_ld8(lane_base + TC_LO + (col0 - kRegCols), lw);
-          tmem_wait_ld();
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int col = n0 + col0 + q;
-            if (col < p.Np)
-              P[(int64_t)col * p.Mp + row] = make_float2(__uint_as_float(hi[q]), __uint_as_float(lw[q]));
+          for (int c = 0; c < 8; ++c) {
+            const int col = n0 + 8 * blk + c;
+            if (col < p.Np) P[(int64_t)col * p.Mp + row] = make_float2(hi[i][c], lo[i][c]);
           }
         }
       }
@@ -778,8 +794,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
-  // no CTA leaves while a CTA of its cluster may still address its shared memory
-  if (p.cl > 1) cluster_sync_all();
 }
 
 // Digit extraction with integer operations only (the FP64 pipe of this part is 1/64 of the
@@ -1037,16 +1051,11 @@ __global__ void oz_slice_hermitian3_kernel(const zd* Hs, int64_t ldh, int n, int
   }
 }
 
-// Columns of B in the Gauss form: column j of Y gives rows j of Yr, Yi, Yr + Yi; columns
-// j >= m of the padded block are zero (the buffer is cleared first).
-__global__ void oz_slice_cols3_kernel(const zd* Y, int64_t ldy, int n, int m, int S, __nv_bfloat16* B,
+// Columns of B in the Gauss form: column j of Y gives rows j of Yr, Yi, Yr + Yi.
+__global__ void oz_slice_cols3_kernel(const zd* Y, int64_t ldy, int n, int S, __nv_bfloat16* B,
                                       int64_t sliceB, int64_t zstride, int Kp, int Np, int* eB,
                                       int lower_half) {
   const int j = blockIdx.x;
-  if (j >= m) {
-    if (threadIdx.x == 0) eB[j] = eB[Np + j] = eB[2 * Np + j] = 0;
-    return;
-  }
   const zd* y = Y + (int64_t)j * ldy;
   // lower_half: as oz_slice_cols_kernel (zero above the diagonal, half of the diagonal entry)
   auto entry = [&](int k) -> zd {
@@ -1190,35 +1199,22 @@ int choose_oz_splits(int tiles, int total_kb, size_t cap_elems, int64_t tile_ele
 }
 
 // Split count for the tcgen05 kernel: split y takes k-blocks [y per, (y + 1) per) of every
-// tile, or (short K) a range of slice pairs.  Modelled CTA time in k-block units: every
-// (panel, pair) chunk costs at least the drain of one accumulator (about 3 k-blocks of
-// streaming time), plus a pipeline fill; the launch time is that times the number of waves
-// of one CTA per SM.
-int choose_tc_splits(int tiles, int nkb, int npairs, size_t cap_elems, int64_t tile_elems, int* pair_split) {
+// tile.  Modelled time in clocks: a K-block costs its tensor work (2 w clocks per slice pair)
+// or its bytes at 36 per clock, a CTA about 5000 more (pipeline fill, last drain, partial
+// sums), and the launch is that times the waves of one CTA per SM; every split adds a write
+// and a read of the partial sums (16 bytes each, about 2800 bytes per clock over the GPU).
+int choose_tc_splits(int tiles, int nz, int nkb, int S, int w, size_t cap_elems, int64_t prod_elems) {
   const int sms = sm_count();
+  const double kb_cost = std::max(S * (S + 1) * (double)w, S * (TC_A_BYTES + 128.0 * w) / 36.0);
   int best = 1;
   double best_cost = 1e300;
-  *pair_split = 0;
-  for (int S = 1; S <= std::min(nkb, 64); ++S) {
-    if ((size_t)S * (size_t)tile_elems > cap_elems) break;
-    const int per = (nkb + S - 1) / S;
-    double cta = 6.0;
-    for (int k0 = 0; k0 < per; k0 += OZ_CHUNK_KB)
-      cta += (double)npairs * std::max(3, std::min(OZ_CHUNK_KB, per - k0));
-    const int64_t units = (int64_t)tiles * S;
-    const double cost = (double)((units + sms - 1) / sms) * cta;
-    if (cost < best_cost * 0.999) { best_cost = cost; best = S; }
-  }
-  // short K (a single panel): splitting the slice pairs gives more CTAs than splitting K
-  if (nkb <= OZ_CHUNK_KB) {
-    for (int S = 2; S <= npairs; ++S) {
-      if ((size_t)S * (size_t)tile_elems > cap_elems) break;
-      const int pp = (npairs + S - 1) / S;
-      const double cta = 6.0 + (double)pp * std::max(3, nkb);
-      const int64_t units = (int64_t)tiles * ((npairs + pp - 1) / pp);
-      const double cost = (double)((units + sms - 1) / sms) * cta;
-      if (cost < best_cost * 0.999) { best_cost = cost; best = (npairs + pp - 1) / pp; *pair_split = 1; }
-    }
+  for (int sp = 1; sp <= std::min(nkb, 64); ++sp) {
+    if ((size_t)sp * (size_t)prod_elems > cap_elems) break;
+    const int per = (nkb + sp - 1) / sp;
+    const int64_t units = (int64_t)tiles * nz * sp;
+    const double cost = (double)((units + sms - 1) / sms) * (per * kb_cost + 5000.0) +
+                        16.0 * (double)sp * nz * (double)prod_elems / 2800.0;
+    if (cost < best_cost * 0.999) { best_cost = cost; best = sp; }
   }
   return best;
 }
@@ -1230,27 +1226,25 @@ int choose_tc_splits(int tiles, int nkb, int npairs, size_t cap_elems, int64_t t
 // product shape, shared by all contexts of the process (batch workers tune from several host
 // threads).  Environment variable CHFSI_OZ_AUTOTUNE=0 keeps the wave model's choice.
 struct TuneKey {
-  int Mp, Np, Kp, S, a_lower, c_lower, group, b_box_rows, cl, ngroups, b_tri, nz;
+  int Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz;
   bool operator<(const TuneKey& o) const {
-    const int a[12] = {Mp, Np, Kp, S, a_lower, c_lower, group, b_box_rows, cl, ngroups, b_tri, nz};
-    const int b[12] = {o.Mp, o.Np, o.Kp, o.S, o.a_lower, o.c_lower, o.group, o.b_box_rows, o.cl, o.ngroups,
-                       o.b_tri, o.nz};
-    return std::lexicographical_compare(a, a + 12, b, b + 12);
+    const int a[9] = {Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz};
+    const int b[9] = {o.Mp, o.Np, o.Kp, o.S, o.a_lower, o.c_lower, o.w, o.b_tri, o.nz};
+    return std::lexicographical_compare(a, a + 9, b, b + 9);
   }
 };
 static std::mutex g_tune_mu;
-static std::map<TuneKey, std::pair<int, int>> g_tune;
-static bool tune_lookup(const TuneKey& k, int* splits, int* pair_split) {
+static std::map<TuneKey, int> g_tune;
+static bool tune_lookup(const TuneKey& k, int* splits) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(k);
   if (it == g_tune.end()) return false;
-  *splits = it->second.first;
-  *pair_split = it->second.second;
+  *splits = it->second;
   return true;
 }
-static void tune_store(const TuneKey& k, int splits, int pair_split) {
+static void tune_store(const TuneKey& k, int splits) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tune[k] = {splits, pair_split};
+  g_tune[k] = splits;
 }
 static bool oz_autotune() {
   static const bool v = [] {
@@ -1274,49 +1268,13 @@ bool oz_use_tcgen05() {
   }();
   return tc;
 }
-// Slice groups sharing one A tile per stage (tcgen05 kernel, blocks up to 96 columns wide);
-// CHFSI_OZ_GROUPS=0 issues one pair per stage instead.
-static bool oz_grouped_pairs() {
-  static const bool grouped = [] {
-    const char* v = std::getenv("CHFSI_OZ_GROUPS");
-    return !(v && std::strcmp(v, "0") == 0);
-  }();
-  return grouped;
-}
-// Largest cluster of CTAs sharing the B tiles of the tcgen05 kernel by multicast: environment
-// variable CHFSI_OZ_CLUSTER (1, 2 or 4; default 1: measured slower on the n = 9300 workload,
-// whose launches are bound by the bytes in flight per SM rather than by the L2 stream).
-static int oz_cluster_max() {
-  static const int v = [] {
-    const char* e = std::getenv("CHFSI_OZ_CLUSTER");
-    const int c = e ? std::atoi(e) : 1;
-    return c >= 4 ? 4 : (c >= 2 ? 2 : 1);
-  }();
-  return v;
-}
-// Order of the tiles over blockIdx.x: environment variable CHFSI_OZ_ORDER ("col": the column
-// tiles of a row tile next to each other; default "row").
-static bool oz_col_major_order() {
-  static const bool v = [] {
-    const char* e = std::getenv("CHFSI_OZ_ORDER");
-    return e && std::strcmp(e, "col") == 0;
-  }();
-  return v;
-}
-// Smallest TMA ring a slice group may leave (its B box grows with the group): environment
-// variable CHFSI_OZ_GROUP_MIN_STAGES, default 4, clamped to [2, TC_MAX_STAGES].
-static int oz_group_min_stages() {
-  static const int v = [] {
-    const char* e = std::getenv("CHFSI_OZ_GROUP_MIN_STAGES");
-    return e ? std::max(2, std::min(TC_MAX_STAGES, std::atoi(e))) : 4;
-  }();
-  return v;
-}
-
-// 2-D bf16 tensor map over `rows` rows of `inner` elements (row pitch inner * 2 bytes),
-// boxes of 64 elements x box_rows rows, 128-byte swizzle (the layout the tcgen05
-// descriptors expect).
-static bool encode_bf16_map(CUtensorMap* map, const void* ptr, int inner, uint64_t rows, int box_rows) {
+// 3-D bf16 tensor map over `slices` slices of `rows` rows of `inner` elements (row pitch
+// `pitch`, slice pitch `slice` elements), boxes of 64 elements x box_rows rows x box_slices
+// slices, 128-byte swizzle (the layout the tcgen05 descriptors expect).  inner and rows are the
+// operand's true extents: the padding of K and of the last tile is filled with zeros by the
+// copy, so the slice buffers need no clearing.
+static bool encode_bf16_map(CUtensorMap* map, const void* ptr, int inner, int pitch, int rows, int64_t slice,
+                            int slices, int box_rows, int box_slices) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   static std::once_flag once;
   std::call_once(once, [] {
@@ -1327,11 +1285,11 @@ static bool encode_bf16_map(CUtensorMap* map, const void* ptr, int inner, uint64
       encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   });
   if (!encode) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)inner * 2};
-  cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides,
+  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)slices};
+  cuuint64_t strides[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)slice * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows, (cuuint32_t)box_slices};
+  cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides,
                             box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
@@ -1339,7 +1297,6 @@ static bool encode_bf16_map(CUtensorMap* map, const void* ptr, int inner, uint64
 int oz_padded_k(int n) { return ((2 * n + OZ_BK - 1) / OZ_BK) * OZ_BK; }
 int oz_padded_m(int n) { return ((2 * n + OZ_BM - 1) / OZ_BM) * OZ_BM; }
 int oz_padded_n(int m) {
-  // tcgen05: multiples of 32 columns, so that a B box splits into four 8-row-aligned shares
   return oz_use_tcgen05() ? ((m + 31) / 32) * 32 : ((m + OZ_BN - 1) / OZ_BN) * OZ_BN;
 }
 
@@ -1368,9 +1325,8 @@ cudaError_t oz_slice_a(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, i
     return cudaErrorInvalidValue;
   a.S = S; a.M = M; a.K = K; a.Mp = Mp; a.Kp = Kp; a.nz = 1;
   a.slice = (int64_t)Mp * Kp;
-  // zero the padding (rows >= 2M, columns >= 2K)
-  cudaError_t e = cudaMemsetAsync(a.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * a.slice, s);
-  if (e != cudaSuccess) return e;
+  // zero the padding (rows >= 2M, columns >= 2K) that the mma.sync kernel reads
+  if (!oz_use_tcgen05()) CK_OZ(cudaMemsetAsync(a.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * a.slice, s));
   if (op == OPC) {
     // op(A) = X^H: row i of op(A) is conj(column i of X), contiguous (X is K x M)
     oz_slice_hermitian_kernel<<<M, 256, 0, s>>>(X, ldx, K, S, a.ptr, a.slice, Kp, a.e);
@@ -1387,13 +1343,13 @@ cudaError_t oz_slice_b(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, i
   if (Np > b.Np_max || Kp > b.Kp_max || S > b.S_max || S < 1 || N <= 0) return cudaErrorInvalidValue;
   b.S = S; b.N = N; b.Np = Np; b.Kp = Kp; b.nz = 1;
   b.slice = (int64_t)Np * Kp;
-  cudaError_t e = cudaMemsetAsync(b.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * b.slice, s);
-  if (e != cudaSuccess) return e;
+  const bool pad = !oz_use_tcgen05();  // the mma.sync kernel reads the padding
+  if (pad) CK_OZ(cudaMemsetAsync(b.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * b.slice, s));
   if (op == OPC) {
     // op(B) = X^H (X is N x K): column j = conj(row j of X)
     CK_OZ(slice_rows(X, ldx, N, K, S, 1, b.ptr, b.slice, Kp, b.e, s));
   } else {
-    oz_slice_cols_kernel<<<Np, 256, 0, s>>>(X, ldx, K, N, S, b.ptr, b.slice, Kp, b.e, lower_half);
+    oz_slice_cols_kernel<<<pad ? Np : N, 256, 0, s>>>(X, ldx, K, N, S, b.ptr, b.slice, Kp, b.e, lower_half);
   }
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
@@ -1428,144 +1384,91 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     tp.a_lower = a_lower;
     tp.b_tri = b_tri;
     tp.c_lower = c_lower;
+    tp.S = S;
     tp.nkb = Kp / OZ_BK;
     tp.tiles_m = Mp / TC_BM;
     tp.Mp = Mp;
     tp.Np = Np;
-    tp.n_real = m;
     tp.part = oz.part;
     tp.status = oz.status;
-    tp.nz = nz;
     tp.kfac = nz > 1 ? 1 : 2;
-    tp.a_zrows = nz > 1 ? a.S * Mp : 0;
-    tp.b_zrows = nz > 1 ? b.S * Np : 0;
+    tp.a_zslices = nz > 1 ? a.S : 0;
+    tp.b_zslices = nz > 1 ? b.S : 0;
+    tp.chunk_kb = tc_chunk_kb(S);
     // first-level waits: the context's bound (a test hook) or the default; the waits that
     // let issued copies and MMAs finish after an abort always use the default
     tp.spin_limit = oz.wait_limit > 0 ? oz.wait_limit : kMbarSpinLimit;
-    // group size (see the kernel's header): tensor memory holds 2 g accumulators of the
-    // block's width rounded up to 32 columns plus the high words, the B box is at most 256
-    // rows, and the ring keeps at least oz_group_min_stages() stages
-    int G = 1;
-    tp.acc_stride = TC_ACC1;
-    if (Np <= TC_GROUP_MAX_N && oz_grouped_pairs()) {
-      const int w = ((Np + 31) / 32) * 32;
-      G = std::min({S, TC_GROUP_MAX, (512 / w - 1) / 2, 256 / Np});
-      while (G > 1 && TC_SMEM_BUDGET / (TC_A_BYTES + G * Np * TC_BK * 2) < oz_group_min_stages()) --G;
-      if (G > 1) tp.acc_stride = w;
-    }
-    tp.group = G;
-    tp.ngroups = 0;
-    for (int si = 1; si <= S; ++si)
-      for (int t0 = 1; si + t0 <= S + 1; t0 += G) {
-        tp.gs[tp.ngroups] = (unsigned char)(si - 1);
-        tp.gt[tp.ngroups] = (unsigned char)(t0 - 1);
-        tp.gc[tp.ngroups] = (unsigned char)std::min(G, S + 2 - si - t0);
-        ++tp.ngroups;
-      }
+    // column tiles: as few as cover the block, of equal width (rounded up to 16 columns).  The
+    // A slices dominate a K-block's bytes, so fewer and wider tiles win over less padding
+    tp.tiles_n = (m + TC_W - 1) / TC_W;
+    tp.w = (((m + tp.tiles_n - 1) / tp.tiles_n + 15) / 16) * 16;
+    // neighbouring CTAs share A: groups of up to 16 column tiles, so that the CTAs resident at
+    // one time (152) cover about 10 row tiles x 16 column tiles of a wide product
+    tp.raster = std::min(tp.tiles_n, 16);
+    const int tiles = tp.tiles_m * tp.tiles_n;
+    const int b_stage = S * tp.w * TC_BK * 2;
+    // rings: two B stages (more while a B stage is small against the A tiles of a K-block), the
+    // rest of the shared memory for A tiles (at least the slices of region 0 stay resident)
+    tp.nb = 2;
+    while (tp.nb < TC_MAX_B && (tp.nb + 1) * b_stage + std::min(2 * S, TC_MAX_A) * TC_A_BYTES <= TC_SMEM_BUDGET)
+      ++tp.nb;
+    tp.na = std::min(TC_MAX_A, (TC_SMEM_BUDGET - tp.nb * b_stage) / TC_A_BYTES);
+    const int levels_per_region = TC_REGION / tp.w;
+    if (tp.na < (S > levels_per_region ? levels_per_region + 1 : 2)) return cudaErrorInvalidValue;
     CUtensorMap mapA, mapB;
-    // The B box is min(Np, TC_BN) rows high (g Np for groups of g); a last tile or group
-    // narrower than that reads rows past its slices (the next slice, the buffer's spare rows:
-    // the allocation holds at least TC_BN rows, or the fill past the map's last row) that
-    // the MMAs never use, since their N covers only the tile's own columns.
-    tp.b_box_rows = G > 1 ? G * Np : std::min(Np, TC_BN);
-    // Cluster of cl CTAs on consecutive row tiles sharing each B box (each loads b_box_rows /
-    // cl rows, a multiple of 8 so that every share starts on a 1024-byte swizzle atom); the
-    // single-CTA launch when the context shortens its waits (the timeout test exercises that
-    // launch's unwinding) or the grid has too few row tiles.
-    tp.cl = 1;
-    if (oz.wait_limit == 0 && oz_cluster_max() > 1)
-      for (int c = oz_cluster_max(); c >= 2; c /= 2)
-        if (tp.tiles_m >= 2 * c && tp.b_box_rows % (8 * c) == 0) {
-          tp.cl = c;
-          break;
-        }
-    tp.tiles_m_pad = ((tp.tiles_m + tp.cl - 1) / tp.cl) * tp.cl;
-    tp.col_major_order = (tp.cl == 1 && oz_col_major_order()) ? 1 : 0;
-    const int tiles = tp.tiles_m_pad * ((Np + TC_BN - 1) / TC_BN);
-    int model_pair_split = 0;
-    const size_t part_cap = oz.part_elems / (size_t)nz;  // partials of each of the nz products
-    const int model_splits =
-        choose_tc_splits(tiles, tp.nkb, tp.ngroups, part_cap, (int64_t)Mp * Np, &model_pair_split);
-    const uint64_t b_rows = std::max<uint64_t>((uint64_t)nz * b.S * Np, (uint64_t)TC_BN);
-    if ((int64_t)b_rows * Kp > b.elems) return cudaErrorInvalidValue;
-    if (!encode_bf16_map(&mapA, a.ptr, Kp, (uint64_t)nz * a.S * Mp, TC_BM) ||
-        !encode_bf16_map(&mapB, b.ptr, Kp, b_rows, tp.b_box_rows / tp.cl))
+    const int kr = nz > 1 ? a.K : 2 * a.K;  // real k extent of both operands
+    if (!encode_bf16_map(&mapA, a.ptr, kr, Kp, nz > 1 ? a.M : 2 * a.M, a.slice, nz * a.S, TC_BM, 1) ||
+        !encode_bf16_map(&mapB, b.ptr, kr, Kp, m, b.slice, nz * b.S, tp.w, S))
       return cudaErrorInvalidValue;
-    const int b_stage = tp.b_box_rows * TC_BK * 2;
-    tp.stages = std::min(TC_MAX_STAGES, TC_SMEM_BUDGET / (TC_A_BYTES + b_stage));
-    const size_t smem = 1024 + (size_t)tp.stages * (TC_A_BYTES + b_stage) + 256;
+    const size_t smem = 1024 + (size_t)tp.na * TC_A_BYTES + (size_t)tp.nb * b_stage + 512;
     // once per process (the library drives one device per process)
     static const cudaError_t tc_attr = cudaFuncSetAttribute(
-        oz_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + TC_SMEM_BUDGET + 256);
+        oz_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + TC_SMEM_BUDGET + 512);
     if (tc_attr != cudaSuccess) return tc_attr;
-    auto launch = [&](int sp, int ps) -> cudaError_t {
+    auto launch = [&](int sp) -> cudaError_t {
       tp.splits = sp;
-      tp.pair_split = ps;
-      if (tp.cl > 1) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(tiles, sp, nz);
-        cfg.blockDim = dim3(TC_THREADS);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = tp.cl;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        cudaError_t le = cudaLaunchKernelEx(&cfg, oz_gemm_tc_kernel, mapA, mapB, tp);
-        if (le != cudaSuccess) return le;
-      } else {
-        oz_gemm_tc_kernel<<<dim3(tiles, sp, nz), TC_THREADS, smem, s>>>(mapA, mapB, tp);
-      }
+      oz_gemm_tc_kernel<<<dim3(tiles, sp, nz), TC_THREADS, smem, s>>>(mapA, mapB, tp);
       CHFSI_COUNT_LAUNCH();
       return cudaGetLastError();
     };
     // split count: the wave model's choice, or the fastest of a few candidates around it,
     // measured on the first product of each shape and kept for the process (autotuner)
-    int best_splits = model_splits, best_ps = model_pair_split;
-    const TuneKey key{Mp, Np, Kp, S, a_lower, c_lower, tp.group, tp.b_box_rows, tp.cl, tp.ngroups, b_tri, nz};
-    if (oz_autotune() && !tune_lookup(key, &best_splits, &best_ps)) {
+    const size_t part_cap = oz.part_elems / (size_t)nz;  // partials of each of the nz products
+    const int model_splits = choose_tc_splits(tiles, nz, tp.nkb, S, tp.w, part_cap, (int64_t)Mp * Np);
+    splits = model_splits;
+    const TuneKey key{Mp, Np, Kp, S, a_lower, c_lower, tp.w, b_tri, nz};
+    if (oz_autotune() && !tune_lookup(key, &splits)) {
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-        std::vector<std::pair<int, int>> cand;
-        const int limit_k = model_pair_split ? tp.ngroups : std::min(tp.nkb, 64);
+        std::vector<int> cand;
         for (int num : {2, 3, 4, 6, 8}) {  // model x {1/2, 3/4, 1, 3/2, 2}
-          const int sp = std::max(1, std::min(limit_k, (model_splits * num + 2) / 4));
+          const int sp = std::max(1, std::min(std::min(tp.nkb, 64), (model_splits * num + 2) / 4));
           if ((size_t)sp * (size_t)((int64_t)Mp * Np) > part_cap) continue;
-          if (model_pair_split) {
-            const int pp = (tp.ngroups + sp - 1) / sp;   // groups per split: the grid uses ceil
-            const int eff = (tp.ngroups + pp - 1) / pp;
-            if (std::find(cand.begin(), cand.end(), std::make_pair(eff, 1)) == cand.end()) cand.push_back({eff, 1});
-          } else if (std::find(cand.begin(), cand.end(), std::make_pair(sp, 0)) == cand.end()) {
-            cand.push_back({sp, 0});
-          }
+          if (std::find(cand.begin(), cand.end(), sp) == cand.end()) cand.push_back(sp);
         }
         cudaEvent_t t0, t1;
         if (cudaEventCreate(&t0) != cudaSuccess || cudaEventCreate(&t1) != cudaSuccess) return cudaGetLastError();
         float best_ms = 1e30f;
-        for (const auto& c : cand) {
+        for (const int c : cand) {
           cudaEventRecord(t0, s);
-          e = launch(c.first, c.second);
+          e = launch(c);
           if (e != cudaSuccess) break;
           cudaEventRecord(t1, s);
           e = cudaEventSynchronize(t1);
           if (e != cudaSuccess) break;
           float ms = 0.f;
           cudaEventElapsedTime(&ms, t0, t1);
-          if (ms < best_ms) { best_ms = ms; best_splits = c.first; best_ps = c.second; }
+          if (ms < best_ms) { best_ms = ms; splits = c; }
         }
         cudaEventDestroy(t0);
         cudaEventDestroy(t1);
         if (e != cudaSuccess) return e;
-        tune_store(key, best_splits, best_ps);
+        tune_store(key, splits);
       }
     }
-    splits = best_splits;
     if ((size_t)splits * (size_t)nz * (size_t)Mp * (size_t)Np > oz.part_elems) return cudaErrorInvalidValue;
     if (ev_gemm_begin) cudaEventRecord(ev_gemm_begin, s);
-    e = launch(best_splits, best_ps);
+    e = launch(splits);
     if (ev_gemm_end) cudaEventRecord(ev_gemm_end, s);
     if (e != cudaSuccess) return e;
   } else {
@@ -1632,8 +1535,6 @@ static cudaError_t oz_slice_a3(OzA& a, int op, const zd* X, int64_t ldx, int M, 
   a.S = S; a.M = M; a.K = K; a.Mp = Mp; a.Kp = Kp; a.nz = 3;
   a.slice = (int64_t)Mp * Kp;
   const int64_t zstride = (int64_t)S * a.slice;
-  cudaError_t e = cudaMemsetAsync(a.ptr, 0, sizeof(__nv_bfloat16) * (size_t)3 * zstride, s);
-  if (e != cudaSuccess) return e;
   if (op == OPC) {
     oz_slice_hermitian3_kernel<<<M, 256, 0, s>>>(X, ldx, K, S, a.ptr, a.slice, zstride, Kp, Mp, a.e);
     CHFSI_COUNT_LAUNCH();
@@ -1657,13 +1558,11 @@ static cudaError_t oz_slice_b3(OzB& b, int op, const zd* X, int64_t ldx, int K, 
                                cudaStream_t s, int lower_half) {
   const int Np = oz_padded_n(N);
   if (S > b.S_max || S < 1 || N <= 0 || K <= 0 || Np > b.Np_max ||
-      (int64_t)3 * S * std::max(Np, TC_BN) * Kp > b.elems)
+      (int64_t)3 * S * Np * Kp > b.elems)
     return cudaErrorInvalidValue;
   b.S = S; b.N = N; b.Np = Np; b.Kp = Kp; b.nz = 3;
   b.slice = (int64_t)Np * Kp;
   const int64_t zstride = (int64_t)S * b.slice;
-  cudaError_t e = cudaMemsetAsync(b.ptr, 0, sizeof(__nv_bfloat16) * (size_t)3 * zstride, s);
-  if (e != cudaSuccess) return e;
   if (op == OPC) {
     const int groups = (N + 31) / 32, kchunks = (K + 31) / 32;
     oz_row_exponents3_kernel<<<groups, 256, 0, s>>>(X, ldx, N, K, 1, b.e, Np);
@@ -1673,16 +1572,9 @@ static cudaError_t oz_slice_b3(OzB& b, int op, const zd* X, int64_t ldx, int K, 
     oz_slice_rows3_kernel<<<dim3(groups, (K + chunk - 1) / chunk), 256, 0, s>>>(
         X, ldx, N, K, S, 1, b.ptr, b.slice, zstride, Kp, b.e, Np, chunk);
     CHFSI_COUNT_LAUNCH();
-    // exponents of the padded columns j >= N
-    if (Np > N) {
-      e = cudaMemsetAsync(b.e + N, 0, sizeof(int) * (size_t)(Np - N), s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(b.e + Np + N, 0, sizeof(int) * (size_t)(Np - N), s);
-      if (e == cudaSuccess) e = cudaMemsetAsync(b.e + 2 * Np + N, 0, sizeof(int) * (size_t)(Np - N), s);
-      if (e != cudaSuccess) return e;
-    }
     return cudaGetLastError();
   }
-  oz_slice_cols3_kernel<<<Np, 256, 0, s>>>(X, ldx, K, N, S, b.ptr, b.slice, zstride, Kp, Np, b.e, lower_half);
+  oz_slice_cols3_kernel<<<N, 256, 0, s>>>(X, ldx, K, S, b.ptr, b.slice, zstride, Kp, Np, b.e, lower_half);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -1745,13 +1637,13 @@ cudaError_t oz_alloc(OzWorkspace& oz, int n_max, int blk_max, int S_max) {
   const int cols = std::max(n_max, blk_max);
   oz.B.S_max = S_max;
   oz.B.Kp_max = oz_padded_k(n_max);
-  // covers both kernels' paddings and at least one full B box of the tcgen05 kernel
-  oz.B.Np_max = ((std::max(cols, TC_BN) + OZ_BN - 1) / OZ_BN) * OZ_BN;
+  // covers both kernels' paddings
+  oz.B.Np_max = ((std::max(cols, TC_W) + OZ_BN - 1) / OZ_BN) * OZ_BN;
   // the Gauss form holds three K x N parts (K padded to 64 complex entries) per slice, the
   // embedding one 2K-row part
   const int64_t kp1 = ((n_max + OZ_BK - 1) / OZ_BK) * OZ_BK;
   oz.B.elems = std::max<int64_t>((int64_t)S_max * oz.B.Np_max * oz.B.Kp_max,
-                                 (int64_t)3 * S_max * std::max(oz.B.Np_max, TC_BN) * kp1);
+                                 (int64_t)3 * S_max * oz.B.Np_max * kp1);
   e = cudaMalloc((void**)&oz.B.ptr, sizeof(__nv_bfloat16) * (size_t)oz.B.elems);
   if (e != cudaSuccess) return e;
   e = cudaMalloc((void**)&oz.B.e, sizeof(int) * (size_t)3 * oz.B.Np_max);
