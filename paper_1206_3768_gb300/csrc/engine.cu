@@ -203,10 +203,13 @@ int gemm_auto(chfsi_ctx* ctx, const GemmDesc& g) {
 // inverse): in mixed mode the large ones run as 8-slice digit products (error about 2^-56 of
 // the operands' row and column scales, below the FP64 GEMM bound; the zero k-blocks of a
 // triangular left or right operand are skipped), the rest in FP64.
-int gemm_factor(chfsi_ctx* ctx, const GemmDesc& g) {
+bool factor_digits(const chfsi_ctx* ctx, const GemmDesc& g) {
   const double work = (double)g.M * g.N * g.K;
   const bool square_c = !g.lowerC || g.M == g.N;
-  if (ctx->opts.precision == 1 && work >= 16777216.0 && square_c) {
+  return ctx->opts.precision == 1 && work >= 16777216.0 && square_c;
+}
+int gemm_factor(chfsi_ctx* ctx, const GemmDesc& g) {
+  if (factor_digits(ctx, g)) {
     CK(oz_gemm(g.opA, g.A, g.lda, g.opB, g.B, g.ldb, g.M, g.N, g.K, 8, g.alpha, g.beta, g.Cin, g.ldcin,
                g.gamma, g.D, g.ldd, g.C, g.ldc, g.triA == 1, g.lowerC, ctx->ws.oz, ctx->stream, g.triB));
     return CHFSI_OK;
@@ -229,6 +232,8 @@ GemmDesc gd(int M, int N, int K, const zd* A, int64_t lda, int opA, const zd* B,
 // Panel width of the blocked factorisations (measured: 256-column panels made the n = 9300
 // workload's reduction phase slower, 2.90 s against 2.81 s per 20-problem step).
 constexpr int NB = 128;
+// Outer panel of the Cholesky factorisation.
+constexpr int NB2 = 512;
 // Digit slices of the FP64-level products in mixed mode (reduction, Rayleigh-Ritz, Gram and
 // rotation products, back-transforms): 7 slices leave an error of about 2^-49 (2e-15)
 // relative to the row and column scales, four orders of magnitude below the 1e-10 bar.
@@ -242,29 +247,48 @@ struct GaussScope {
   ~GaussScope() { oz.gauss = saved; }
 };
 
-// In-place blocked right-looking Cholesky on the lower triangle of L (n x n).  Its digit
-// products keep the real embedding (the factor's errors reach every later step).
-int blocked_cholesky(chfsi_ctx* ctx, zd* L, int64_t ld, int n, int nb = NB) {
+// In-place blocked right-looking Cholesky on the lower triangle of L (n x n), in two levels: NB
+// columns at a time within outer panels of nb2 columns, the matrix to the right of an outer
+// panel updated once per panel.  That update reads and writes all that is left of the matrix and
+// slices the panel again, so fewer and deeper ones are cheaper.  Its digit products keep the
+// real embedding (the factor's errors reach every later step).
+int blocked_cholesky(chfsi_ctx* ctx, zd* L, int64_t ld, int n, int nb = NB, int nb2 = NB2) {
   Workspace& ws = ctx->ws;
   GaussScope gs(ws.oz, 0);
-  for (int k0 = 0; k0 < n; k0 += nb) {
-    const int kb = std::min(nb, n - k0);
-    zd* L11 = L + k0 + (int64_t)k0 * ld;
-    CK(small_cholesky(L11, ld, kb, 0, 0, 0.0, nullptr, nullptr, ws.status, ws.status + 1, k0,
-                      ctx->stream));
-    const int r = n - k0 - kb;
+  for (int p0 = 0; p0 < n; p0 += nb2) {
+    const int p1 = std::min(n, p0 + nb2);
+    for (int k0 = p0; k0 < p1; k0 += nb) {
+      const int kb = std::min(nb, p1 - k0);
+      zd* L11 = L + k0 + (int64_t)k0 * ld;
+      CK(panel_cholesky(L11, ld, kb, ws.status, ws.status + 1, k0, ctx->stream));
+      const int r = n - k0 - kb;
+      if (r <= 0) break;
+      // L21 = A21 L11^{-H}
+      CK(trinv_lower(L11, ld, ws.Rt, ws.blk_max, kb, ctx->stream));
+      zd* A21 = L + (k0 + kb) + (int64_t)k0 * ld;
+      GemmDesc g = gd(r, kb, kb, A21, ld, OPN, ws.Rt, ws.blk_max, OPC, A21, ld);
+      g.triB = 1;
+      const bool in_place = factor_digits(ctx, g);  // operands are sliced before the result is written
+      if (!in_place) { g.C = ws.Z; g.ldc = r; }
+      CKS(gemm_factor(ctx, g));
+      if (!in_place)
+        CK(cudaMemcpy2DAsync(A21, ld * sizeof(zd), ws.Z, r * sizeof(zd), r * sizeof(zd), kb,
+                             cudaMemcpyDeviceToDevice, ctx->stream));
+      // the rest of the outer panel: A(:, k0 + kb .. p1) -= L21 L21(0 .. c)^H
+      const int c = p1 - k0 - kb;
+      if (c > 0) {
+        zd* Ac = L + (k0 + kb) + (int64_t)(k0 + kb) * ld;
+        GemmDesc u = gd(r, c, kb, A21, ld, OPN, A21, ld, OPC, Ac, ld, -1.0);
+        u.beta = 1.0; u.Cin = Ac; u.ldcin = ld;
+        CKS(gemm_factor(ctx, u));
+      }
+    }
+    // A22 -= Lp Lp^H (lower), Lp the outer panel below its diagonal block
+    const int r = n - p1;
     if (r <= 0) break;
-    // L21 = A21 L11^{-H}
-    CK(trinv_lower(L11, ld, ws.Rt, ws.blk_max, kb, ctx->stream));
-    zd* A21 = L + (k0 + kb) + (int64_t)k0 * ld;
-    GemmDesc g = gd(r, kb, kb, A21, ld, OPN, ws.Rt, ws.blk_max, OPC, ws.Z, r);
-    g.triB = 1;
-    CKS(gemm_factor(ctx, g));
-    CK(cudaMemcpy2DAsync(A21, ld * sizeof(zd), ws.Z, r * sizeof(zd), r * sizeof(zd), kb,
-                         cudaMemcpyDeviceToDevice, ctx->stream));
-    // A22 -= L21 L21^H (lower)
-    zd* A22 = L + (k0 + kb) + (int64_t)(k0 + kb) * ld;
-    GemmDesc h = gd(r, r, kb, A21, ld, OPN, A21, ld, OPC, A22, ld, -1.0);
+    zd* Lp = L + p1 + (int64_t)p0 * ld;
+    zd* A22 = L + p1 + (int64_t)p1 * ld;
+    GemmDesc h = gd(r, r, p1 - p0, Lp, ld, OPN, Lp, ld, OPC, A22, ld, -1.0);
     h.beta = 1.0; h.Cin = A22; h.ldcin = ld; h.lowerC = 1;
     CKS(gemm_factor(ctx, h));
   }
@@ -272,26 +296,35 @@ int blocked_cholesky(chfsi_ctx* ctx, zd* L, int64_t ld, int n, int nb = NB) {
   return CHFSI_OK;
 }
 
-// X = L^{-1} (n x n, lower) by block rows: X_II = inv(L_II),
-// X[I, 0:I] = -X_II (L[I, 0:I] X[0:I, 0:I]).
-int blocked_trinv(chfsi_ctx* ctx, const zd* L, int64_t ld, zd* X, int64_t ldx, int n, int nb = NB) {
+// The blocks below the diagonal of X = L^{-1}, the NB x NB diagonal blocks of X being there:
+// [X11 0; X21 X22] with X21 = -X22 (L21 X11), L11 the largest NB 2^k rows below n.  T: n x n
+// scratch.  Halving makes the products square and slices each part of X once per level, where
+// block rows would slice all of X above for every NB rows.
+int trinv_halves(chfsi_ctx* ctx, const zd* L, int64_t ld, zd* X, int64_t ldx, zd* T, int64_t ldt, int n) {
+  if (n <= NB) return CHFSI_OK;
+  int n1 = NB;
+  while (2 * n1 < n) n1 *= 2;
+  const int n2 = n - n1;
+  const zd* L21 = L + n1;
+  zd* X21 = X + n1;
+  zd* X22 = X + n1 + (int64_t)n1 * ldx;
+  CKS(trinv_halves(ctx, L, ld, X, ldx, T, ldt, n1));
+  CKS(trinv_halves(ctx, L + n1 + (int64_t)n1 * ld, ld, X22, ldx, T, ldt, n2));
+  GemmDesc g = gd(n2, n1, n1, L21, ld, OPN, X, ldx, OPN, T, ldt);
+  g.triB = 2;
+  CKS(gemm_factor(ctx, g));
+  GemmDesc h = gd(n2, n1, n2, X22, ldx, OPN, T, ldt, OPN, X21, ldx, -1.0);
+  h.triA = 1;
+  return gemm_factor(ctx, h);
+}
+
+// X = L^{-1} (n x n, lower): the inverses of all diagonal blocks in one launch, then by halves.
+int blocked_trinv(chfsi_ctx* ctx, const zd* L, int64_t ld, zd* X, int64_t ldx, int n) {
   Workspace& ws = ctx->ws;
   GaussScope gs(ws.oz, 0);  // the embedding, as in blocked_cholesky
   CK(cudaMemset2DAsync(X, ldx * sizeof(zd), 0, n * sizeof(zd), n, ctx->stream));
-  for (int k0 = 0; k0 < n; k0 += nb) {
-    const int kb = std::min(nb, n - k0);
-    CK(trinv_lower(L + k0 + (int64_t)k0 * ld, ld, X + k0 + (int64_t)k0 * ldx, ldx, kb, ctx->stream));
-    if (k0 == 0) continue;
-    // Zt = L[I, 0:k0] X[0:k0, 0:k0]  (kb x k0), X lower => op(B)(k, j) = 0 for k < j
-    GemmDesc g = gd(kb, k0, k0, L + k0, ld, OPN, X, ldx, OPN, ws.Z, kb);
-    g.triB = 2;
-    CKS(gemm_factor(ctx, g));
-    // X[I, 0:k0] = -X_II Zt, X_II lower
-    GemmDesc h = gd(kb, k0, kb, X + k0 + (int64_t)k0 * ldx, ldx, OPN, ws.Z, kb, OPN, X + k0, ldx, -1.0);
-    h.triA = 1;
-    CKS(gemm_factor(ctx, h));
-  }
-  return CHFSI_OK;
+  CK(trinv_lower_blocks(L, ld, X, ldx, n, NB, ctx->stream));
+  return trinv_halves(ctx, L, ld, X, ldx, ws.T, ws.n_max, n);
 }
 
 // Hs = Linv Af Linv^H.  split: the two products use split-BF16 tensor-core products

@@ -79,6 +79,11 @@ cudaError_t small_cholesky(zd* G, int64_t ldg, int m, int scale, int shift_on_fa
                            int info_base, cudaStream_t s, int* shift_flag = nullptr);
 // X = L^{-1} for an m x m lower-triangular L (strict upper of X zeroed).  X != L.
 cudaError_t trinv_lower(const zd* L, int64_t ldl, zd* X, int64_t ldx, int m, cudaStream_t s);
+// Inverses of the m-row diagonal blocks of the n x n lower-triangular L into X's blocks.
+cudaError_t trinv_lower_blocks(const zd* L, int64_t ldl, zd* X, int64_t ldx, int n, int m, cudaStream_t s);
+// Cholesky of one diagonal block (m <= 128) in place on the lower triangle (the strict upper
+// triangle is left alone); a failed pivot sets DEV_NOTPD and info = min(info, info_base + pivot).
+cudaError_t panel_cholesky(zd* G, int64_t ldg, int m, int* status, int* info, int info_base, cudaStream_t s);
 // One pass of the mixed-precision re-orthonormalisation (Y <- Y T) from G = Y^H Y (lower):
 // a first-order Loewdin step in FP64 when ||G - I||_F <= 1e-3 (flags[0] = 1 once that norm
 // is <= 1e-8), else an FP32 Cholesky QR step on the scaled Gram (shift on breakdown), whose
