@@ -482,7 +482,7 @@ int filter_block(chfsi_ctx* ctx, const zd* H, int64_t ldh, int n, int m, zd** Ya
     if (slices > 0) {
       // split-BF16 tensor-core product with the same fused recurrence epilogue
       CK(oz_filter_product(cur, ld, n, mk, slices, al, be, cur, ld, k >= 2 ? ga : 0.0, out, ld, out,
-                           ld, ws.oz, ctx->stream, gb, ge));
+                           ld, ws.oz, ctx->stream, gb, ge, /*keys_in=*/k > 1, /*keys_out=*/k < dmax));
       if (st) {
         // slice-pair flops the kernel issues: the 2n x 2n real embedding, or the Gauss form's
         // three real n x n products

@@ -224,6 +224,10 @@ struct OzWorkspace {
   int* status = nullptr;            // device status word for bounded-wait timeouts
   long long wait_limit = 0;         // polls of a first-level mbarrier wait (0: the default)
   int gauss = 1;                    // the Gauss form is allowed for the current products
+  // scale keys (see the slicing kernels) of up to three parts of an operand's columns or rows: two
+  // buffers, one read by a product's slicing while its epilogue fills the other
+  unsigned* key[2] = {nullptr, nullptr};
+  int key_cur = 0, key_np = 0;      // buffer and stride of the last epilogue's keys
 };
 bool oz_use_tcgen05();
 int oz_padded_k(int n);
@@ -232,15 +236,11 @@ int oz_padded_n(int m);
 int64_t oz_pair_count(int S);
 cudaError_t oz_alloc(OzWorkspace& oz, int n_max, int blk_max, int S_max);
 void oz_free(OzWorkspace& oz);
-// Digit slices of op(A) = X (op N: rows of X, M x K) or X^H (op C: conj columns of X, K x M).
-cudaError_t oz_slice_a(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, int S, cudaStream_t s);
-// Digit slices of op(B) = X (op N: columns, K x N) or X^H (op C: conj rows of X, N x K).
-cudaError_t oz_slice_b(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, int S, int Kp,
-                       cudaStream_t s, int lower_half = 0);
 cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double beta, const zd* Cin,
                        int64_t ldcin, double gamma, const zd* D, int64_t ldd, zd* out, int64_t ldo,
                        int a_lower, int c_lower, OzWorkspace& oz, cudaStream_t s,
-                       cudaEvent_t ev_gemm_begin = nullptr, cudaEvent_t ev_gemm_end = nullptr, int b_tri = 0);
+                       cudaEvent_t ev_gemm_begin = nullptr, cudaEvent_t ev_gemm_end = nullptr, int b_tri = 0,
+                       unsigned* key_out = nullptr);
 // Slices of the Hermitian Hs into oz.H (once per problem).
 cudaError_t oz_slice_hermitian(const zd* Hs, int64_t ldh, int n, int S, OzWorkspace& oz,
                                cudaStream_t s);
@@ -248,7 +248,8 @@ cudaError_t oz_slice_hermitian(const zd* Hs, int64_t ldh, int n, int S, OzWorksp
 cudaError_t oz_filter_product(const zd* Y, int64_t ldy, int n, int m, int S, double alpha,
                               double beta, const zd* Cin, int64_t ldcin, double gamma, const zd* D,
                               int64_t ldd, zd* out, int64_t ldo, OzWorkspace& oz, cudaStream_t s,
-                              cudaEvent_t ev_gemm_begin = nullptr, cudaEvent_t ev_gemm_end = nullptr);
+                              cudaEvent_t ev_gemm_begin = nullptr, cudaEvent_t ev_gemm_end = nullptr,
+                              bool keys_in = false, bool keys_out = false);
 // General split product on the scratch operands.
 cudaError_t oz_gemm(int opA, const zd* A, int64_t lda, int opB, const zd* B, int64_t ldb, int M, int N,
                     int K, int S, double alpha, double beta, const zd* Cin, int64_t ldcin, double gamma,

@@ -224,39 +224,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const OzParams p
     }
 }
 
-// Complex epilogue: C(i, j) = 2^{eA(i)+eB(j)} (sum_s P[s](2i, j), sum_s P[s](2i+1, j)),
-// out = alpha C + beta Cin + gamma D (out may alias Cin or D element-wise).  The partial
-// sums are FP64 (pairs == 0) or double-float (hi, lo) pairs of FP32 (pairs != 0), which are
-// summed over the splits in double-float arithmetic and converted to FP64 once.
-__global__ void oz_epilogue_kernel(const double* part, int splits, int Mp, int Np, const int* eA,
-                                   const int* eB, int n, int m, double alpha, double beta,
-                                   const zd* Cin, int64_t ldcin, double gamma, const zd* D,
-                                   int64_t ldd, zd* out, int64_t ldo, int lower, int pairs) {
+// Complex epilogue of the mma.sync kernel: C(i, j) = 2^{eA(i)+eB(j)} (sum_s P[s](2i, j), sum_s P[s](2i+1,
+// j)), out = alpha C + beta Cin + gamma D (out may alias Cin or D element-wise), from FP64 partials.
+__global__ void oz_mma_epilogue_kernel(const double* part, int splits, int Mp, int Np, const int* eA,
+                                       const int* eB, int n, int m, double alpha, double beta,
+                                       const zd* Cin, int64_t ldcin, double gamma, const zd* D,
+                                       int64_t ldd, zd* out, int64_t ldo, int lower) {
   const int64_t total = (int64_t)n * m;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e % n), j = (int)(e / n);
     if (lower && j > i) continue;
     double re = 0.0, im = 0.0;
-    if (pairs) {
-      float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-      for (int s = 0; s < splits; ++s) {
-        const float4 v = *reinterpret_cast<const float4*>(part + (int64_t)s * Mp * Np +
+    for (int s = 0; s < splits; ++s) {
+      const double2 v = *reinterpret_cast<const double2*>(part + (int64_t)s * Mp * Np +
                                                           (int64_t)j * Mp + 2 * i);
-        two_sum_acc(rh, rl, v.x);
-        rl += v.y;
-        two_sum_acc(ih, il, v.z);
-        il += v.w;
-      }
-      re = (double)rh + (double)rl;
-      im = (double)ih + (double)il;
-    } else {
-      for (int s = 0; s < splits; ++s) {
-        const double2 v = *reinterpret_cast<const double2*>(part + (int64_t)s * Mp * Np +
-                                                            (int64_t)j * Mp + 2 * i);
-        re += v.x;
-        im += v.y;
-      }
+      re += v.x;
+      im += v.y;
     }
     // the kernel applied the slice-level scales 2^{-7(s+t)}; the row and column scales remain
     const int ex = eA[i] + eB[j];
@@ -266,7 +250,6 @@ __global__ void oz_epilogue_kernel(const double* part, int splits, int Mp, int N
     out[i + (int64_t)j * ldo] = o;
   }
 }
-
 
 // ============================================================================ tcgen05 path
 // The same digit products on the 5th-generation tensor cores (tcgen05.mma, bf16 inputs, FP32
@@ -796,391 +779,362 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-// Digit extraction with integer operations only (the FP64 pipe of this part is 1/64 of the
-// FP32 rate, so shifting the 53-bit significand is much cheaper than FP64 arithmetic).
-// |x| is a non-negative double: its bit pattern orders like its value.
-__device__ __forceinline__ unsigned long long abs_bits(double x) {
-  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+// ============================================================================ digit slices
+// Digits come from integer operations on the bit patterns (an FP64 instruction occupies an SM
+// quarter for 64 clocks).
+//
+// Key of |x|: its high word, the lowest bit set when the low word is not zero.  Keys order like
+// the exponents and are zero for zero only, so a column's scale is a maximum of 32-bit words.
+__device__ __forceinline__ unsigned abs_key(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7FFFFFFFu) | (__double2loint(x) != 0 ? 1u : 0u);
 }
-// smallest e with max < 2^e, from the bit pattern of max (0 for max == 0)
-__device__ __forceinline__ int exponent_from_bits(unsigned long long mb) {
-  if (mb == 0) return 0;
-  const int E = (int)(mb >> 52);
+// smallest e with |x| < 2^e for every x of the maximal key (0 for zero)
+__device__ __forceinline__ int exponent_of_key(unsigned key) {
+  if (key == 0u) return 0;
+  const int E = (int)(key >> 20);
   return (E ? E : 1) - 1022;
 }
-// Balanced digits of x (|x| < 2^e), computed with integer operations: y = |x| 2^{-e} is
-// rounded to 7S fractional bits, split into base-128 digits, and re-centred from the least
-// significant end (a digit >= 64 becomes digit - 128 with a carry into the next one), so
-// that digits 2..S lie in [-64, 63] and digit 1 in [0, 129]; the sign of x is applied to all.
-// Then |x - 2^e sum_k d_k 2^{-7k}| <= 2^{e-7S-1}, and the dropped slice pairs of a product
-// carry digits of both signs (they largely cancel).  Every digit is exact in bf16.
-__device__ __forceinline__ void digits(double x, int e, int S, __nv_bfloat16* out, int64_t stride) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int E = (int)((bits >> 52) & 0x7FF);
-  const bool neg = (bits >> 63) != 0;
-  unsigned long long mant = (bits & 0xFFFFFFFFFFFFFull) | (E ? (1ull << 52) : 0ull);
-  const int Eu = (E ? E : 1) - 1075;  // x = mant * 2^Eu
-  const int sh_last = e - Eu - OZ_BETA * S;
-  if (sh_last >= 1 && sh_last <= 63) mant += 1ull << (sh_last - 1);  // round half up (magnitude)
-  int d[8];
+// Balanced digits of x (|x| < 2^e): y = |x| 2^{-e} rounded to 7S fractional bits is sum_k d_k 128^-k
+// with d_2 .. d_S in [-64, 63] and d_1 in [0, 129]; the sign of x is applied to all.  Adding 64 at
+// every place from the second on makes the places plain base-128 digits d_k + 64, so the word
+// below holds all of them, place k at bit 7 (8 - k), without a carry chain.  Then |x - 2^e sum_k d_k
+// 2^{-7k}| <= 2^{e-7S-1}, and the dropped slice pairs of a product carry digits of both signs (they
+// largely cancel).  Every digit is exact in bf16.
+struct DigitWord {
+  unsigned long long z;
+  unsigned sign;  // sign bit of x
+};
+__device__ __forceinline__ unsigned long long digit_centre(int S) {  // 64 at places 2 .. S
+  unsigned long long c = 0;
 #pragma unroll
-  for (int k = 1; k <= 8; ++k) {
-    if (k > S) break;
-    const int sh = e - Eu - OZ_BETA * k;  // right shift that leaves digit k in the low bits
-    unsigned long long w;
-    if (sh >= 64) w = 0ull;
-    else if (sh >= 0) w = mant >> sh;
-    else w = mant << (-sh);
-    d[k - 1] = (k == 1) ? (int)w : (int)(w & 127ull);
-  }
+  for (int k = 2; k <= 8; ++k)
+    if (k <= S) c |= 64ull << (7 * (8 - k));
+  return c;
+}
+__device__ __forceinline__ DigitWord digit_word(double x, int e, int S, unsigned long long centre) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  const int E = (int)((hi >> 20) & 0x7FFu);
+  const unsigned long long mant =
+      ((unsigned long long)((hi & 0xFFFFFu) | (E ? 0x100000u : 0u)) << 32) | (unsigned)__double2loint(x);
+  const int sh = e - ((E ? E : 1) - 1075) - OZ_BETA * S;  // x = mant 2^(E - 1075); drop sh bits of it
+  unsigned long long y;
+  if (sh >= 1) y = sh <= 63 ? (mant + (1ull << (sh - 1))) >> sh : 0ull;  // round half up (magnitude)
+  else y = mant << -sh;
+  DigitWord w;
+  w.z = (y << (OZ_BETA * (8 - S))) + centre;
+  w.sign = hi & 0x80000000u;
+  return w;
+}
+// bits of the FP32 value of digit k (1 ..): the place put into the significand of 2^23, less 2^23 (+ 64)
+__device__ __forceinline__ unsigned digit_float_bits(const DigitWord& w, int k) {
+  const unsigned u = k == 1 ? (unsigned)(w.z >> 49) : ((unsigned)(w.z >> (7 * (8 - k))) & 127u);
+  return __float_as_uint(__uint_as_float(0x4B000000u | u) - (k == 1 ? 8388608.f : 8388672.f)) ^ w.sign;
+}
+// two neighbouring bf16 digits (the high halves of their FP32 values)
+__device__ __forceinline__ unsigned digit_pair(const DigitWord& a, const DigitWord& b, int k) {
+  return __byte_perm(digit_float_bits(a, k), digit_float_bits(b, k), 0x7632);
+}
+// digits of two neighbouring entries into S slices (out: 4-byte aligned)
+__device__ __forceinline__ void store_digits(double a, double b, int e, int S, unsigned long long centre,
+                                             __nv_bfloat16* out, int64_t slice) {
+  const DigitWord wa = digit_word(a, e, S, centre), wb = digit_word(b, e, S, centre);
 #pragma unroll
-  for (int k = 8; k >= 2; --k) {
-    if (k > S) continue;
-    if (d[k - 1] >= 64) {
-      d[k - 1] -= 128;
-      d[k - 2] += 1;
-    }
-  }
+  for (int k = 1; k <= 8; ++k)
+    if (k <= S) *reinterpret_cast<unsigned*>(out + (int64_t)(k - 1) * slice) = digit_pair(wa, wb, k);
+}
+// digits of two neighbouring complex entries, (re, im) interleaved (out: 8-byte aligned)
+__device__ __forceinline__ void store_digits_ri(double ar, double ai, double br, double bi, int e, int S,
+                                                unsigned long long centre, __nv_bfloat16* out, int64_t slice) {
+  const DigitWord w0 = digit_word(ar, e, S, centre), w1 = digit_word(ai, e, S, centre);
+  const DigitWord w2 = digit_word(br, e, S, centre), w3 = digit_word(bi, e, S, centre);
 #pragma unroll
-  for (int k = 1; k <= 8; ++k) {
-    if (k > S) break;
-    const float v = (float)(neg ? -d[k - 1] : d[k - 1]);
-    out[(int64_t)(k - 1) * stride] = __float2bfloat16_rn(v);
-  }
+  for (int k = 1; k <= 8; ++k)
+    if (k <= S)
+      *reinterpret_cast<uint2*>(out + (int64_t)(k - 1) * slice) =
+          make_uint2(digit_pair(w0, w1, k), digit_pair(w2, w3, k));
 }
 
-__device__ unsigned long long block_max_bits(unsigned long long v) {
-  __shared__ unsigned long long sh[32];
-  __shared__ unsigned long long res;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
-    v = t > v ? t : v;
-  }
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    unsigned long long t = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0ull;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long u = __shfl_xor_sync(0xffffffffu, t, o);
-      t = u > t ? u : t;
-    }
-    if (lane == 0) res = t;
-  }
-  __syncthreads();
-  const unsigned long long r = res;
-  __syncthreads();
-  return r;
-}
+__device__ __forceinline__ unsigned warp_max(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
 
-// A-side slices of the real embedding of Hermitian Hs: one CTA per complex row i.
-// Row i of Hs is conj(column i), read contiguously.  Real rows 2i, 2i+1; columns 2k, 2k+1:
-//   [ Re h  -Im h ]      h = Hs(i, k) = conj(Hs(k, i))
-//   [ Im h   Re h ]
-__global__ void oz_slice_hermitian_kernel(const zd* Hs, int64_t ldh, int n, int S,
-                                          __nv_bfloat16* A, int64_t sliceA, int Kp, int* eA) {
-  // (n = K: the length of column i of X, i.e. of row i of op(A) = X^H)
-  const int i = blockIdx.x;
-  const zd* col = Hs + (int64_t)i * ldh;
-  unsigned long long mx = 0ull;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd h = col[k];
-    const unsigned long long a = abs_bits(h.x), b = abs_bits(h.y);
-    mx = a > mx ? a : mx;
-    mx = b > mx ? b : mx;
-  }
-  mx = block_max_bits(mx);
-  const int e = exponent_from_bits(mx);
-  if (threadIdx.x == 0) eA[i] = e;
-  __nv_bfloat16* r0 = A + (int64_t)(2 * i) * Kp;
-  __nv_bfloat16* r1 = r0 + Kp;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd hc = col[k];
-    const double re = hc.x, im = -hc.y;  // H(i,k) = conj(Hs(k,i))
-    digits(re, e, S, r0 + 2 * k, sliceA);
-    digits(-im, e, S, r0 + 2 * k + 1, sliceA);
-    digits(im, e, S, r1 + 2 * k, sliceA);
-    digits(re, e, S, r1 + 2 * k + 1, sliceA);
-  }
-}
+// Operand layouts.  Embedding (one part): B column j = (re, im) of column j interleaved; A rows 2i,
+// 2i + 1 = [Re, -Im], [Im, Re] interleaved.  Gauss form (three real products instead of the 2n x 2n
+// embedding): Hs Y = (Hr Yr - Hi Yi) + i ((Hr + Hi)(Yr + Yi) - Hr Yr - Hi Yi), parts re, im, re + im
+// with a scale per row or column each, slices [part][s][row][k], scales [part][row].  The sums
+// are formed in FP64 (one rounding) before the digits are taken.
+enum { FORM_EMBED_B = 0, FORM_EMBED_A = 1, FORM_GAUSS = 2 };
 
-
-// Slices from the ROWS of a general complex matrix X (rows x cols, column-major), in two
-// kernels: the row scales need a full pass over each row, and a row is strided in memory,
-// so 32-row groups are read column by column (coalesced) to find the row exponents; the
-// digits are then written by CTAs that each take one 32-row group and one range of columns
-// (transposed through shared memory), so that thin matrices still spread over the GPU.
-//   mode 0 (A operand, real embedding): rows 2r, 2r+1 of A^ = [Re x, -Im x], [Im x, Re x]
-//   mode 1 (B operand of X^H): column r of B^ = conj(row r of X) = [Re x, -Im x]
-__global__ void oz_row_exponents_kernel(const zd* X, int64_t ldx, int rows, int cols, int* e_out) {
-  __shared__ unsigned long long red[8][32];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  const int r = blockIdx.x * 32 + tx;
-  unsigned long long mx = 0ull;
-  if (r < rows)
-    for (int k = ty; k < cols; k += 8) {
-      const zd v = X[r + (int64_t)k * ldx];
-      const unsigned long long a = abs_bits(v.x), b = abs_bits(v.y);
-      mx = a > mx ? a : mx;
-      mx = b > mx ? b : mx;
-    }
-  red[ty][tx] = mx;
-  __syncthreads();
-  if (ty == 0 && r < rows) {
-    unsigned long long m2 = red[0][tx];
-    for (int j = 1; j < 8; ++j) m2 = red[j][tx] > m2 ? red[j][tx] : m2;
-    e_out[r] = exponent_from_bits(m2);
-  }
-}
-
-__global__ void oz_slice_rows_kernel(const zd* X, int64_t ldx, int rows, int cols, int S, int mode,
-                                     __nv_bfloat16* out, int64_t slice_stride, int Kp, const int* e_row,
-                                     int chunk) {
-  __shared__ int ex[32];
-  __shared__ zd tile[32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  const int r0 = blockIdx.x * 32;
-  if (ty == 0) ex[tx] = (r0 + tx < rows) ? e_row[r0 + tx] : 0;
-  __syncthreads();
-  const int k_end = min(cols, (int)(blockIdx.y + 1) * chunk);
-  for (int k0 = blockIdx.y * chunk; k0 < k_end; k0 += 32) {
-    for (int rr = ty; rr < 32; rr += 8) {
-      const int gr = r0 + tx, gk = k0 + rr;  // read column gk, rows r0..r0+31 (coalesced)
-      tile[rr][tx] = (gr < rows && gk < k_end) ? X[gr + (int64_t)gk * ldx] : zmk(0.0, 0.0);
-    }
-    __syncthreads();
-    for (int rr = ty; rr < 32; rr += 8) {  // write row r0 + rr, columns k0 + tx (coalesced)
-      const int gr = r0 + rr, gk = k0 + tx;
-      if (gr < rows && gk < k_end) {
-        const zd v = tile[tx][rr];
-        const int e = ex[rr];
-        if (mode == 0) {
-          __nv_bfloat16* o0 = out + (int64_t)(2 * gr) * Kp + 2 * gk;
-          __nv_bfloat16* o1 = o0 + Kp;
-          digits(v.x, e, S, o0, slice_stride);
-          digits(-v.y, e, S, o0 + 1, slice_stride);
-          digits(v.y, e, S, o1, slice_stride);
-          digits(v.x, e, S, o1 + 1, slice_stride);
-        } else {
-          __nv_bfloat16* o0 = out + (int64_t)gr * Kp + 2 * gk;
-          digits(v.x, e, S, o0, slice_stride);
-          digits(-v.y, e, S, o0 + 1, slice_stride);
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// B-side slices of Y^ (the n x m complex block read as a 2n x m real array): one CTA per
-// column j; columns j >= m of the padded block are zero.
-// lower_half: column j of the operand is column j of Y below the diagonal, half of Y(j, j)
-// on it and zero above (the lower part L_h of a Hermitian Y = L_h + L_h^H).
-__global__ void oz_slice_cols_kernel(const zd* Y, int64_t ldy, int n, int m, int S,
-                                     __nv_bfloat16* B, int64_t sliceB, int Kp, int* eB, int lower_half) {
-  const int j = blockIdx.x;
-  __nv_bfloat16* col = B + (int64_t)j * Kp;
-  if (j >= m) {
-    for (int k = threadIdx.x; k < Kp; k += blockDim.x)
-      for (int s = 0; s < S; ++s) col[s * sliceB + k] = __float2bfloat16_rn(0.f);
-    if (threadIdx.x == 0) eB[j] = 0;
-    return;
-  }
-  const zd* y = Y + (int64_t)j * ldy;
-  auto entry = [&](int k) -> zd {
-    zd v = y[k];
+// Entry k of column j of the operand: conjugated (rows of a Hermitian or of X^H), or its lower half
+// (zero above the diagonal, half of the diagonal entry: the lower part L_h of Y = L_h + L_h^H).
+struct ColumnSource {
+  const zd* Y;
+  int64_t ldy;
+  int n, conj, lower_half;
+  __device__ __forceinline__ zd at(int j, int k) const {
+    if (k >= n) return zmk(0.0, 0.0);
+    zd v = Y[k + (int64_t)j * ldy];
+    if (conj) v.y = __hiloint2double(__double2hiint(v.y) ^ (int)0x80000000, __double2loint(v.y));
     if (lower_half) {
       if (k < j) v = zmk(0.0, 0.0);
       else if (k == j) v = zmk(0.5 * v.x, 0.5 * v.y);
     }
     return v;
-  };
-  unsigned long long mx = 0ull;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd v = entry(k);
-    const unsigned long long a = abs_bits(v.x), b = abs_bits(v.y);
-    mx = a > mx ? a : mx;
-    mx = b > mx ? b : mx;
   }
-  mx = block_max_bits(mx);
-  const int e = exponent_from_bits(mx);
-  if (threadIdx.x == 0) eB[j] = e;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd v = entry(k);
-    digits(v.x, e, S, col + 2 * k, sliceB);
-    digits(v.y, e, S, col + 2 * k + 1, sliceB);
-  }
-}
+};
 
-// Gauss form of the complex product (three real products instead of the 2n x 2n real
-// embedding): Hs Y = (Hr Yr - Hi Yi) + i ((Hr + Hi)(Yr + Yi) - Hr Yr - Hi Yi).  Operand z of
-// A is Hr, Hi, Hr + Hi (z = 0, 1, 2) with its own power-of-two scale per row, operand z of B
-// is Yr, Yi, Yr + Yi with its own scale per column; slices [z][s][row][k], scales [z][row].
-// The sums Hr + Hi and Yr + Yi are formed in FP64 (one rounding) before the digits are taken.
-// Rows of A: row i of H = conj(column i of Hs) (Hs Hermitian), read contiguously.
-__global__ void oz_slice_hermitian3_kernel(const zd* Hs, int64_t ldh, int n, int S, __nv_bfloat16* A,
-                                           int64_t sliceA, int64_t zstride, int Kp, int Mp, int* eA) {
-  const int i = blockIdx.x;
-  const zd* col = Hs + (int64_t)i * ldh;
-  unsigned long long m0 = 0ull, m1 = 0ull, m2 = 0ull;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd h = col[k];
-    const double hr = h.x, hi = -h.y, hs = hr + hi;
-    const unsigned long long a = abs_bits(hr), b = abs_bits(hi), c = abs_bits(hs);
-    m0 = a > m0 ? a : m0;
-    m1 = b > m1 ? b : m1;
-    m2 = c > m2 ? c : m2;
+// Keys of the columns' parts: key[part * stride + j], raised by atomicMax (cleared before).  Grid:
+// (row chunks, columns).
+__global__ void oz_col_keys_kernel(const ColumnSource src, int parts, unsigned* key, int stride, int chunk) {
+  const int j = blockIdx.y, k1 = min(src.n, (int)(blockIdx.x + 1) * chunk);
+  unsigned m0 = 0, m1 = 0, m2 = 0;
+  for (int k = blockIdx.x * chunk + threadIdx.x; k < k1; k += blockDim.x) {
+    const zd v = src.at(j, k);
+    m0 = max(m0, abs_key(v.x));
+    m1 = max(m1, abs_key(v.y));
+    if (parts == 3) m2 = max(m2, abs_key(v.x + v.y));
   }
-  const int e0 = exponent_from_bits(block_max_bits(m0));
-  const int e1 = exponent_from_bits(block_max_bits(m1));
-  const int e2 = exponent_from_bits(block_max_bits(m2));
-  if (threadIdx.x == 0) {
-    eA[i] = e0;
-    eA[Mp + i] = e1;
-    eA[2 * Mp + i] = e2;
-  }
-  __nv_bfloat16* r0 = A + (int64_t)i * Kp;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd h = col[k];
-    const double hr = h.x, hi = -h.y;
-    digits(hr, e0, S, r0 + k, sliceA);
-    digits(hi, e1, S, r0 + zstride + k, sliceA);
-    digits(hr + hi, e2, S, r0 + 2 * zstride + k, sliceA);
-  }
-}
-
-// Columns of B in the Gauss form: column j of Y gives rows j of Yr, Yi, Yr + Yi.
-__global__ void oz_slice_cols3_kernel(const zd* Y, int64_t ldy, int n, int S, __nv_bfloat16* B,
-                                      int64_t sliceB, int64_t zstride, int Kp, int Np, int* eB,
-                                      int lower_half) {
-  const int j = blockIdx.x;
-  const zd* y = Y + (int64_t)j * ldy;
-  // lower_half: as oz_slice_cols_kernel (zero above the diagonal, half of the diagonal entry)
-  auto entry = [&](int k) -> zd {
-    zd v = y[k];
-    if (lower_half) {
-      if (k < j) v = zmk(0.0, 0.0);
-      else if (k == j) v = zmk(0.5 * v.x, 0.5 * v.y);
+  if (parts == 1) m0 = max(m0, m1);
+  m0 = warp_max(m0);
+  m1 = warp_max(m1);
+  m2 = warp_max(m2);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(key + j, m0);
+    if (parts == 3) {
+      atomicMax(key + stride + j, m1);
+      atomicMax(key + 2 * stride + j, m2);
     }
-    return v;
-  };
-  unsigned long long m0 = 0ull, m1 = 0ull, m2 = 0ull;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd v = entry(k);
-    const unsigned long long a = abs_bits(v.x), b = abs_bits(v.y), c = abs_bits(v.x + v.y);
-    m0 = a > m0 ? a : m0;
-    m1 = b > m1 ? b : m1;
-    m2 = c > m2 ? c : m2;
-  }
-  const int e0 = exponent_from_bits(block_max_bits(m0));
-  const int e1 = exponent_from_bits(block_max_bits(m1));
-  const int e2 = exponent_from_bits(block_max_bits(m2));
-  if (threadIdx.x == 0) {
-    eB[j] = e0;
-    eB[Np + j] = e1;
-    eB[2 * Np + j] = e2;
-  }
-  __nv_bfloat16* c0 = B + (int64_t)j * Kp;
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const zd v = entry(k);
-    digits(v.x, e0, S, c0 + k, sliceB);
-    digits(v.y, e1, S, c0 + zstride + k, sliceB);
-    digits(v.x + v.y, e2, S, c0 + 2 * zstride + k, sliceB);
   }
 }
 
-// Gauss-form slices from the ROWS of X (rows x cols, column-major): row r of the operand is
-// row r of X (conj = 0: an A operand) or its conjugate (conj = 1: column r of a B operand
-// op(B) = X^H); the three parts re, im, re + im get a scale per row each (e[z * e_stride + r])
-// and their digits go to out + z * zstride + r * Kp + k.  Same two-kernel scheme as the
-// embedding's row slices.
-__global__ void oz_row_exponents3_kernel(const zd* X, int64_t ldx, int rows, int cols, int conj, int* e_out,
-                                         int e_stride) {
-  __shared__ unsigned long long red[3][8][32];
+// Slices of columns (B operands, and A operands whose rows are conjugated columns).  Grid: (row
+// chunks, columns); each thread takes two neighbouring entries, so that a slice is written four
+// (eight) bytes at a time.  The columns' keys come from the kernel above or from the epilogue
+// that wrote the block; without them (key == nullptr, one chunk) the CTA scans its column first,
+// which is cheaper when there are columns enough to fill the GPU (the second read hits L2).
+// clear: the key words of the same columns that the next epilogue will raise.
+template <int FORM>
+__global__ void oz_slice_cols_kernel(const ColumnSource src, int S, __nv_bfloat16* out, int64_t slice,
+                                     int64_t zstride, int Kp, int* e_out, int e_stride, const unsigned* key,
+                                     unsigned* clear, int chunk) {
+  constexpr int parts = FORM == FORM_GAUSS ? 3 : 1;
+  const int j = blockIdx.y, tid = threadIdx.x;
+  unsigned kz[3] = {0, 0, 0};
+  if (key) {
+#pragma unroll
+    for (int z = 0; z < parts; ++z) kz[z] = key[z * e_stride + j];
+  } else {
+    __shared__ unsigned sh[3][32];
+    for (int k = tid; k < src.n; k += blockDim.x) {
+      const zd v = src.at(j, k);
+      kz[0] = max(kz[0], abs_key(v.x));
+      kz[1] = max(kz[1], abs_key(v.y));
+      if (parts == 3) kz[2] = max(kz[2], abs_key(v.x + v.y));
+    }
+    if (parts == 1) kz[0] = max(kz[0], kz[1]);
+#pragma unroll
+    for (int z = 0; z < parts; ++z) {
+      const unsigned v = warp_max(kz[z]);
+      if ((tid & 31) == 0) sh[z][tid >> 5] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int z = 0; z < parts; ++z) {
+      unsigned v = sh[z][0];
+      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = max(v, sh[z][w]);
+      kz[z] = v;
+    }
+  }
+  int e[3];
+#pragma unroll
+  for (int z = 0; z < parts; ++z) e[z] = exponent_of_key(kz[z]);
+  if (blockIdx.x == 0 && tid == 0) {
+#pragma unroll
+    for (int z = 0; z < parts; ++z) {
+      e_out[z * e_stride + j] = e[z];
+      if (clear) clear[z * e_stride + j] = 0u;
+    }
+  }
+  const unsigned long long centre = digit_centre(S);
+  const int k1 = min(src.n, (int)(blockIdx.x + 1) * chunk);
+  for (int k = blockIdx.x * chunk + 2 * tid; k < k1; k += 2 * blockDim.x) {
+    const zd u = src.at(j, k), v = src.at(j, k + 1);
+    if (FORM == FORM_GAUSS) {
+      __nv_bfloat16* o = out + (int64_t)j * Kp + k;
+      store_digits(u.x, v.x, e[0], S, centre, o, slice);
+      store_digits(u.y, v.y, e[1], S, centre, o + zstride, slice);
+      store_digits(u.x + u.y, v.x + v.y, e[2], S, centre, o + 2 * zstride, slice);
+    } else if (FORM == FORM_EMBED_B) {
+      store_digits_ri(u.x, u.y, v.x, v.y, e[0], S, centre, out + (int64_t)j * Kp + 2 * k, slice);
+    } else {
+      __nv_bfloat16* o = out + (int64_t)(2 * j) * Kp + 2 * k;
+      store_digits_ri(u.x, -u.y, v.x, -v.y, e[0], S, centre, o, slice);
+      store_digits_ri(u.y, u.x, v.y, v.x, e[0], S, centre, o + Kp, slice);
+    }
+  }
+}
+
+// Keys of the ROWS of X (rows x cols, column-major) or of its conjugate: 32-row groups read column by
+// column (coalesced), the columns shared out over blockIdx.y.
+__global__ void oz_row_keys_kernel(const zd* X, int64_t ldx, int rows, int cols, int conj, int parts, unsigned* key,
+                                   int stride) {
+  __shared__ unsigned red[3][8][32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const int r = blockIdx.x * 32 + tx;
-  unsigned long long m0 = 0ull, m1 = 0ull, m2 = 0ull;
+  unsigned m0 = 0, m1 = 0, m2 = 0;
   if (r < rows)
-    for (int k = ty; k < cols; k += 8) {
+    for (int k = blockIdx.y * 8 + ty; k < cols; k += 8 * gridDim.y) {
       const zd v = X[r + (int64_t)k * ldx];
-      const double re = v.x, im = conj ? -v.y : v.y;
-      const unsigned long long a = abs_bits(re), b = abs_bits(im), c = abs_bits(re + im);
-      m0 = a > m0 ? a : m0;
-      m1 = b > m1 ? b : m1;
-      m2 = c > m2 ? c : m2;
+      m0 = max(m0, abs_key(v.x));
+      m1 = max(m1, abs_key(v.y));
+      if (parts == 3) m2 = max(m2, abs_key(conj ? v.x - v.y : v.x + v.y));
     }
+  if (parts == 1) m0 = max(m0, m1);
   red[0][ty][tx] = m0;
   red[1][ty][tx] = m1;
   red[2][ty][tx] = m2;
   __syncthreads();
-  if (ty < 3 && r < rows) {
-    unsigned long long mz = red[ty][0][tx];
-    for (int j = 1; j < 8; ++j) mz = red[ty][j][tx] > mz ? red[ty][j][tx] : mz;
-    e_out[ty * e_stride + r] = exponent_from_bits(mz);
+  if (ty < parts && r < rows) {
+    unsigned m = red[ty][0][tx];
+    for (int w = 1; w < 8; ++w) m = max(m, red[ty][w][tx]);
+    atomicMax(key + ty * stride + r, m);
   }
 }
 
-__global__ void oz_slice_rows3_kernel(const zd* X, int64_t ldx, int rows, int cols, int S, int conj,
-                                      __nv_bfloat16* out, int64_t slice_stride, int64_t zstride, int Kp,
-                                      const int* e_row, int e_stride, int chunk) {
+// Slices of the ROWS of X (or of its conjugate): CTAs take one 32-row group and one range of columns
+// each, 32 x 32 tiles transposed through shared memory, so that thin matrices still spread over
+// the GPU; each thread writes two neighbouring entries.
+template <int FORM>
+__global__ void oz_slice_rows_kernel(const zd* X, int64_t ldx, int rows, int cols, int S, int conj,
+                                     __nv_bfloat16* out, int64_t slice, int64_t zstride, int Kp, int* e_out,
+                                     int e_stride, const unsigned* key, int chunk) {
+  constexpr int parts = FORM == FORM_GAUSS ? 3 : 1;
   __shared__ int ex[3][32];
   __shared__ zd tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const int r0 = blockIdx.x * 32;
-  if (ty < 3) ex[ty][tx] = (r0 + tx < rows) ? e_row[ty * e_stride + r0 + tx] : 0;
-  __syncthreads();
+  if (ty < parts) {
+    const int e = r0 + tx < rows ? exponent_of_key(key[ty * e_stride + r0 + tx]) : 0;
+    ex[ty][tx] = e;
+    if (blockIdx.y == 0 && r0 + tx < rows) e_out[ty * e_stride + r0 + tx] = e;
+  }
+  const unsigned long long centre = digit_centre(S);
   const int k_end = min(cols, (int)(blockIdx.y + 1) * chunk);
   for (int k0 = blockIdx.y * chunk; k0 < k_end; k0 += 32) {
-    for (int rr = ty; rr < 32; rr += 8) {
-      const int gr = r0 + tx, gk = k0 + rr;  // read column gk, rows r0..r0+31 (coalesced)
-      tile[rr][tx] = (gr < rows && gk < k_end) ? X[gr + (int64_t)gk * ldx] : zmk(0.0, 0.0);
+    for (int c = ty; c < 32; c += 8) {
+      const int gr = r0 + tx, gk = k0 + c;  // read column gk, rows r0 .. r0 + 31 (coalesced)
+      zd v = (gr < rows && gk < k_end) ? X[gr + (int64_t)gk * ldx] : zmk(0.0, 0.0);
+      if (conj) v.y = __hiloint2double(__double2hiint(v.y) ^ (int)0x80000000, __double2loint(v.y));
+      tile[c][tx] = v;
     }
     __syncthreads();
-    for (int rr = ty; rr < 32; rr += 8) {  // write row r0 + rr, columns k0 + tx (coalesced)
-      const int gr = r0 + rr, gk = k0 + tx;
-      if (gr < rows && gk < k_end) {
-        const zd v = tile[tx][rr];
-        const double re = v.x, im = conj ? -v.y : v.y;
+    for (int it = threadIdx.x; it < 512; it += 256) {  // row r0 + it / 16, columns k0 + 2 (it % 16) and the next
+      const int rr = it >> 4, c = 2 * (it & 15), gr = r0 + rr, gk = k0 + c;
+      if (gr >= rows || gk >= k_end) continue;
+      const zd u = tile[c][rr], v = tile[c + 1][rr];
+      if (FORM == FORM_GAUSS) {
         __nv_bfloat16* o = out + (int64_t)gr * Kp + gk;
-        digits(re, ex[0][rr], S, o, slice_stride);
-        digits(im, ex[1][rr], S, o + zstride, slice_stride);
-        digits(re + im, ex[2][rr], S, o + 2 * zstride, slice_stride);
+        store_digits(u.x, v.x, ex[0][rr], S, centre, o, slice);
+        store_digits(u.y, v.y, ex[1][rr], S, centre, o + zstride, slice);
+        store_digits(u.x + u.y, v.x + v.y, ex[2][rr], S, centre, o + 2 * zstride, slice);
+      } else if (FORM == FORM_EMBED_B) {
+        store_digits_ri(u.x, u.y, v.x, v.y, ex[0][rr], S, centre, out + (int64_t)gr * Kp + 2 * gk, slice);
+      } else {
+        __nv_bfloat16* o = out + (int64_t)(2 * gr) * Kp + 2 * gk;
+        store_digits_ri(u.x, -u.y, v.x, -v.y, ex[0][rr], S, centre, o, slice);
+        store_digits_ri(u.y, u.x, v.y, v.x, ex[0][rr], S, centre, o + Kp, slice);
       }
     }
     __syncthreads();
   }
 }
 
-// out = alpha (P0 - P1 + i (P2 - P0 - P1)) + beta Cin + gamma D from the split partials of
-// the three real products (double-float pairs, slice scales applied), each scaled by its row
-// and column exponents.
-__global__ void oz_epilogue3_kernel(const float2* part, int splits, int Mp, int Np, const int* eA,
-                                    const int* eB, int n, int m, double alpha, double beta,
-                                    const zd* Cin, int64_t ldcin, double gamma, const zd* D,
-                                    int64_t ldd, zd* out, int64_t ldo, int lower) {
-  const int64_t total = (int64_t)n * m;
-  const int64_t zst = (int64_t)splits * Mp * Np;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e % n), j = (int)(e / n);
-    if (lower && j > i) continue;
-    double v[3];
+// ============================================================================ epilogue
+// (h + l) 2^ex: the exponents are raised in the bit patterns, one FP64 addition is left (FP64
+// conversions and ldexp cost several each, and the epilogue was bound by them).
+__device__ __forceinline__ double widen_scaled(float x, int ex, bool& in_range) {
+  const int f = __float_as_int(x), e = (f >> 23) & 0xFF;
+  const int ne = e - 127 + 1023 + ex;
+  if (e == 0) return 0.0;
+  in_range = ne > 0 && ne < 2047;
+  return __hiloint2double((f & 0x80000000) | (ne << 20) | ((f & 0x7FFFFF) >> 3), f << 29);
+}
+__device__ __forceinline__ double scaled_sum(float h, float l, int ex) {
+  bool ok_h = true, ok_l = true;
+  const double dh = widen_scaled(h, ex, ok_h), dl = widen_scaled(l, ex, ok_l);
+  if (!(ok_h && ok_l)) return ldexp((double)h + (double)l, ex);  // near the ends of the FP64 range
+  return dh + dl;
+}
+
+// out = alpha C + beta Cin + gamma D (out may alias Cin or D element-wise) from the split partials of
+// the tensor-core kernel (double-float pairs, slice scales applied), each scaled by its row and
+// column exponents.  NZ = 1: C(i, j) from rows 2i, 2i + 1 of the embedding; NZ = 3: C = P0 - P1 +
+// i (P2 - P0 - P1) from the Gauss form's three products.  key (optional): the keys of the columns of
+// out, for the slices of the next product (cleared before).  Grid: (row chunks, columns).
+// What bounds it: 13 FP64 instructions an entry on large blocks (n = 9300, m = 320: 195 -> 113 us), the
+// chain of loads on small ones, which is why the splits' loads are issued in groups of four.
+template <int NZ>
+__global__ void __launch_bounds__(256)
+    oz_epilogue_kernel(const float2* part, int splits, int Mp, int Np, const int* eA, const int* eB, int n,
+                       double alpha, double beta, const zd* Cin, int64_t ldcin, double gamma, const zd* D,
+                       int64_t ldd, zd* out, int64_t ldo, int lower, unsigned* key, int key_stride, int rows) {
+  const int64_t prod = (int64_t)Mp * Np, zst = splits * prod;
+  const int i1 = min(n, (int)(blockIdx.x + 1) * rows), j = blockIdx.y;
+  int eb[NZ];
 #pragma unroll
-    for (int z = 0; z < 3; ++z) {
-      float h = 0.f, l = 0.f;
+  for (int z = 0; z < NZ; ++z) eb[z] = eB[z * Np + j];
+  unsigned m0 = 0, m1 = 0, m2 = 0;
+  for (int i = blockIdx.x * rows + threadIdx.x; i < i1; i += 256) {
+    if (lower && j > i) continue;
+    const zd cin = beta != 0.0 ? Cin[i + (int64_t)j * ldcin] : zmk(0.0, 0.0);
+    const zd d = gamma != 0.0 ? D[i + (int64_t)j * ldd] : zmk(0.0, 0.0);
+    zd o;
+    if (NZ == 1) {
+      float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+#pragma unroll 4
       for (int sp = 0; sp < splits; ++sp) {
-        const float2 q = part[z * zst + (int64_t)sp * Mp * Np + (int64_t)j * Mp + i];
-        two_sum_acc(h, l, q.x);
-        l += q.y;
+        const float4 v = *reinterpret_cast<const float4*>(part + sp * prod + (int64_t)j * Mp + 2 * i);
+        two_sum_acc(rh, rl, v.x);
+        rl += v.y;
+        two_sum_acc(ih, il, v.z);
+        il += v.w;
       }
-      v[z] = ldexp((double)h + (double)l, eA[z * Mp + i] + eB[z * Np + j]);
+      const int ex = eA[i] + eb[0];
+      o = zmk(alpha * scaled_sum(rh, rl, ex), alpha * scaled_sum(ih, il, ex));
+    } else {
+      double v[3];
+#pragma unroll
+      for (int z = 0; z < 3; ++z) {
+        float h = 0.f, l = 0.f;
+#pragma unroll 4
+        for (int sp = 0; sp < splits; ++sp) {
+          const float2 q = part[z * zst + sp * prod + (int64_t)j * Mp + i];
+          two_sum_acc(h, l, q.x);
+          l += q.y;
+        }
+        v[z] = scaled_sum(h, l, eA[z * Mp + i] + eb[NZ == 3 ? z : 0]);
+      }
+      o = zmk(alpha * (v[0] - v[1]), alpha * (v[2] - v[0] - v[1]));
     }
-    zd o = zmk(alpha * (v[0] - v[1]), alpha * (v[2] - v[0] - v[1]));
-    if (beta != 0.0) o = zadd(o, zscale(Cin[i + (int64_t)j * ldcin], beta));
-    if (gamma != 0.0) o = zadd(o, zscale(D[i + (int64_t)j * ldd], gamma));
+    if (beta != 0.0) o = zadd(o, zscale(cin, beta));
+    if (gamma != 0.0) o = zadd(o, zscale(d, gamma));
     out[i + (int64_t)j * ldo] = o;
+    if (key) {
+      m0 = max(m0, abs_key(o.x));
+      m1 = max(m1, abs_key(o.y));
+      if (NZ == 3) m2 = max(m2, abs_key(o.x + o.y));
+    }
+  }
+  if (key) {
+    if (NZ == 1) m0 = max(m0, m1);
+    m0 = warp_max(m0);
+    m1 = warp_max(m1);
+    m2 = warp_max(m2);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(key + j, m0);
+      if (NZ == 3) {
+        atomicMax(key + key_stride + j, m1);
+        atomicMax(key + 2 * key_stride + j, m2);
+      }
+    }
   }
 }
 
@@ -1301,25 +1255,98 @@ int oz_padded_n(int m) {
 }
 
 // ---- operands
-// Row exponents, then digits by (32-row group, column range) CTAs: about four CTAs per SM.
-static cudaError_t slice_rows(const zd* X, int64_t ldx, int rows, int cols, int S, int mode, __nv_bfloat16* out,
-                              int64_t slice_stride, int Kp, int* e_out, cudaStream_t s) {
-  const int groups = (rows + 31) / 32, kchunks = (cols + 31) / 32;
-  oz_row_exponents_kernel<<<groups, 256, 0, s>>>(X, ldx, rows, cols, e_out);
-  CHFSI_COUNT_LAUNCH();
-  const int gy = std::max(1, std::min(kchunks, (4 * sm_count() + groups - 1) / groups));
-  const int chunk = 32 * ((kchunks + gy - 1) / gy);
-  oz_slice_rows_kernel<<<dim3(groups, (cols + chunk - 1) / chunk), 256, 0, s>>>(X, ldx, rows, cols, S, mode, out,
-                                                                                slice_stride, Kp, e_out, chunk);
-  return cudaGetLastError();
-}
 #define CK_OZ(expr)                 \
   do {                              \
     cudaError_t e_ = (expr);        \
     if (e_ != cudaSuccess) return e_; \
   } while (0)
 
-cudaError_t oz_slice_a(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, int S, cudaStream_t s) {
+// Where a sliced operand goes: buffer, scales and layout.
+struct SliceDst {
+  __nv_bfloat16* ptr;
+  int64_t slice, zstride;
+  int Kp;
+  int* e;
+  int e_stride, form, S;
+};
+
+// Slices of `cols` columns (length n): keys from `key` if given, else scanned by the slicing CTA when
+// there are two columns or more per SM, else by a kernel of their own over row chunks.
+static cudaError_t slice_cols(const ColumnSource& src, int cols, const SliceDst& d, OzWorkspace& oz, cudaStream_t s,
+                              const unsigned* key = nullptr, unsigned* clear = nullptr) {
+  const int sms = sm_count();
+  int chunk = src.n, gx = 1;
+  if (key || cols < 2 * sms) {
+    gx = std::max(1, std::min((src.n + 511) / 512, (6 * sms + cols - 1) / cols));
+    chunk = ((src.n + gx - 1) / gx + 511) / 512 * 512;
+    gx = (src.n + chunk - 1) / chunk;
+    if (!key) {
+      const int parts = d.form == FORM_GAUSS ? 3 : 1;
+      CK_OZ(cudaMemsetAsync(oz.key[oz.key_cur], 0, sizeof(unsigned) * (size_t)parts * d.e_stride, s));
+      oz_col_keys_kernel<<<dim3(gx, cols), 256, 0, s>>>(src, parts, oz.key[oz.key_cur], d.e_stride, chunk);
+      CHFSI_COUNT_LAUNCH();
+      key = oz.key[oz.key_cur];
+    }
+  }
+  const dim3 grid(gx, cols);
+  if (d.form == FORM_GAUSS)
+    oz_slice_cols_kernel<FORM_GAUSS><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e, d.e_stride,
+                                                          key, clear, chunk);
+  else if (d.form == FORM_EMBED_A)
+    oz_slice_cols_kernel<FORM_EMBED_A><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e,
+                                                            d.e_stride, key, clear, chunk);
+  else
+    oz_slice_cols_kernel<FORM_EMBED_B><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e,
+                                                            d.e_stride, key, clear, chunk);
+  CHFSI_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+
+// Slices of the rows of X (rows x cols) or of its conjugate: keys, then digits by (32-row group, column
+// range) CTAs, about four CTAs per SM each.
+static cudaError_t slice_rows(const zd* X, int64_t ldx, int rows, int cols, int conj, const SliceDst& d,
+                              OzWorkspace& oz, cudaStream_t s) {
+  const int groups = (rows + 31) / 32, kchunks = (cols + 31) / 32, parts = d.form == FORM_GAUSS ? 3 : 1;
+  unsigned* key = oz.key[oz.key_cur];
+  CK_OZ(cudaMemsetAsync(key, 0, sizeof(unsigned) * (size_t)parts * d.e_stride, s));
+  const int gy = std::max(1, std::min(kchunks, (4 * sm_count() + groups - 1) / groups));
+  oz_row_keys_kernel<<<dim3(groups, gy), 256, 0, s>>>(X, ldx, rows, cols, conj, parts, key, d.e_stride);
+  CHFSI_COUNT_LAUNCH();
+  const int chunk = 32 * ((kchunks + gy - 1) / gy);
+  const dim3 grid(groups, (cols + chunk - 1) / chunk);
+  if (d.form == FORM_GAUSS)
+    oz_slice_rows_kernel<FORM_GAUSS><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
+                                                          d.Kp, d.e, d.e_stride, key, chunk);
+  else if (d.form == FORM_EMBED_A)
+    oz_slice_rows_kernel<FORM_EMBED_A><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
+                                                            d.Kp, d.e, d.e_stride, key, chunk);
+  else
+    oz_slice_rows_kernel<FORM_EMBED_B><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
+                                                            d.Kp, d.e, d.e_stride, key, chunk);
+  CHFSI_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+
+// op(A) (M x K) as the A operand.  op = OPC: row i of op(A) is the conjugated column i of X (K x M,
+// contiguous); op = OPN: row i of X (M x K, strided).
+static cudaError_t slice_a_into(OzA& a, int form, int op, const zd* X, int64_t ldx, int M, int K, int S,
+                                OzWorkspace& oz, cudaStream_t s) {
+  const SliceDst d{a.ptr, a.slice, (int64_t)S * a.slice, a.Kp, a.e, a.Mp, form, S};
+  if (op == OPC) return slice_cols(ColumnSource{X, ldx, K, 1, 0}, M, d, oz, s);
+  return slice_rows(X, ldx, M, K, 0, d, oz, s);
+}
+// op(B) (K x N) as the B operand.  op = OPN: column j of X (optionally its lower half); op = OPC: the
+// conjugated row j of X (N x K).
+static cudaError_t slice_b_into(OzB& b, int form, int op, const zd* X, int64_t ldx, int K, int N, int S,
+                                int lower_half, OzWorkspace& oz, cudaStream_t s, const unsigned* key = nullptr,
+                                unsigned* clear = nullptr) {
+  const SliceDst d{b.ptr, b.slice, (int64_t)S * b.slice, b.Kp, b.e, b.Np, form, S};
+  if (op == OPN) return slice_cols(ColumnSource{X, ldx, K, 0, lower_half}, N, d, oz, s, key, clear);
+  return slice_rows(X, ldx, N, K, 1, d, oz, s);
+}
+
+static cudaError_t oz_slice_a(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, int S, OzWorkspace& oz,
+                              cudaStream_t s) {
   const int Kp = oz_padded_k(K), Mp = oz_padded_m(M);
   if (S > a.S_max || S < 1 || Kp > a.Kp_max || Mp > a.Mp_max || M <= 0 || K <= 0)
     return cudaErrorInvalidValue;
@@ -1327,32 +1354,19 @@ cudaError_t oz_slice_a(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, i
   a.slice = (int64_t)Mp * Kp;
   // zero the padding (rows >= 2M, columns >= 2K) that the mma.sync kernel reads
   if (!oz_use_tcgen05()) CK_OZ(cudaMemsetAsync(a.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * a.slice, s));
-  if (op == OPC) {
-    // op(A) = X^H: row i of op(A) is conj(column i of X), contiguous (X is K x M)
-    oz_slice_hermitian_kernel<<<M, 256, 0, s>>>(X, ldx, K, S, a.ptr, a.slice, Kp, a.e);
-  } else {
-    CK_OZ(slice_rows(X, ldx, M, K, S, 0, a.ptr, a.slice, Kp, a.e, s));
-  }
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  return slice_a_into(a, FORM_EMBED_A, op, X, ldx, M, K, S, oz, s);
 }
 
-cudaError_t oz_slice_b(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, int S, int Kp,
-                       cudaStream_t s, int lower_half) {
+static cudaError_t oz_slice_b(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, int S, int Kp, OzWorkspace& oz,
+                              cudaStream_t s, int lower_half = 0, const unsigned* key = nullptr,
+                              unsigned* clear = nullptr) {
   const int Np = oz_padded_n(N);
   if (Np > b.Np_max || Kp > b.Kp_max || S > b.S_max || S < 1 || N <= 0) return cudaErrorInvalidValue;
   b.S = S; b.N = N; b.Np = Np; b.Kp = Kp; b.nz = 1;
   b.slice = (int64_t)Np * Kp;
-  const bool pad = !oz_use_tcgen05();  // the mma.sync kernel reads the padding
-  if (pad) CK_OZ(cudaMemsetAsync(b.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * b.slice, s));
-  if (op == OPC) {
-    // op(B) = X^H (X is N x K): column j = conj(row j of X)
-    CK_OZ(slice_rows(X, ldx, N, K, S, 1, b.ptr, b.slice, Kp, b.e, s));
-  } else {
-    oz_slice_cols_kernel<<<pad ? Np : N, 256, 0, s>>>(X, ldx, K, N, S, b.ptr, b.slice, Kp, b.e, lower_half);
-  }
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  // as in oz_slice_a
+  if (!oz_use_tcgen05()) CK_OZ(cudaMemsetAsync(b.ptr, 0, sizeof(__nv_bfloat16) * (size_t)S * b.slice, s));
+  return slice_b_into(b, FORM_EMBED_B, op, X, ldx, K, N, S, lower_half, oz, s, key, clear);
 }
 
 // out (M x N complex, M = a.M, N = b.N) = alpha op(A) op(B) + beta Cin + gamma D from the
@@ -1361,7 +1375,7 @@ cudaError_t oz_slice_b(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, i
 cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double beta, const zd* Cin,
                        int64_t ldcin, double gamma, const zd* D, int64_t ldd, zd* out, int64_t ldo,
                        int a_lower, int c_lower, OzWorkspace& oz, cudaStream_t s,
-                       cudaEvent_t ev_gemm_begin, cudaEvent_t ev_gemm_end, int b_tri) {
+                       cudaEvent_t ev_gemm_begin, cudaEvent_t ev_gemm_end, int b_tri, unsigned* key_out) {
   const int n = a.M, m = b.N, Kp = a.Kp, Mp = a.Mp, Np = b.Np;
   if (m <= 0 || n <= 0) return cudaSuccess;
   if (S > b.S || S > a.S || S < 1 || a.Kp != b.Kp || a.nz != b.nz) return cudaErrorInvalidValue;
@@ -1499,16 +1513,23 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  const int64_t tot = (int64_t)n * m;
-  const int blocks = (int)std::min<int64_t>(4 * sm_count(), (tot + 255) / 256);
-  if (nz == 3)
-    oz_epilogue3_kernel<<<blocks, 256, 0, s>>>(reinterpret_cast<const float2*>(oz.part), splits, Mp, Np, a.e,
-                                               b.e, n, m, alpha, beta, Cin, ldcin, gamma, D, ldd, out, ldo,
-                                               c_lower);
-  else
-    oz_epilogue_kernel<<<blocks, 256, 0, s>>>(oz.part, splits, Mp, Np, a.e, b.e, n, m, alpha, beta, Cin,
-                                              ldcin, gamma, D, ldd, out, ldo, c_lower,
-                                              oz_use_tcgen05() ? 1 : 0);
+  if (!oz_use_tcgen05()) {
+    const int64_t tot = (int64_t)n * m;
+    const int blocks = (int)std::min<int64_t>(4 * sm_count(), (tot + 255) / 256);
+    oz_mma_epilogue_kernel<<<blocks, 256, 0, s>>>(oz.part, splits, Mp, Np, a.e, b.e, n, m, alpha, beta, Cin, ldcin,
+                                                  gamma, D, ldd, out, ldo, c_lower);
+  } else {
+    // 1024 rows a CTA of 256 threads, 256 while that leaves less than eight CTAs per SM
+    const int rows = (int64_t)((n + 1023) / 1024) * m >= 8 * sm_count() ? 1024 : 256;
+    const dim3 grid((n + rows - 1) / rows, m);
+    const float2* part = reinterpret_cast<const float2*>(oz.part);
+    if (nz == 3)
+      oz_epilogue_kernel<3><<<grid, 256, 0, s>>>(part, splits, Mp, Np, a.e, b.e, n, alpha, beta, Cin, ldcin, gamma, D,
+                                                 ldd, out, ldo, c_lower, key_out, Np, rows);
+    else
+      oz_epilogue_kernel<1><<<grid, 256, 0, s>>>(part, splits, Mp, Np, a.e, b.e, n, alpha, beta, Cin, ldcin, gamma, D,
+                                                 ldd, out, ldo, c_lower, key_out, Np, rows);
+  }
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -1524,81 +1545,68 @@ static bool oz_gauss(const OzWorkspace& oz) {
   return v && oz.gauss && oz_use_tcgen05();
 }
 
-// op(A) (M x K) as the Gauss-form A operand: slices of its real part, imaginary part and
-// their sum, a scale per row of each.  op = OPC: row i is the conjugated column i of X (K x M,
-// contiguous); op = OPN: row i of X (M x K, strided; row slices as the embedding's).
-static cudaError_t oz_slice_a3(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, int S, cudaStream_t s) {
+// The Gauss-form operands: slices of the real part, the imaginary part and their sum, a scale per row
+// (A) or column (B) of each.
+static cudaError_t oz_slice_a3(OzA& a, int op, const zd* X, int64_t ldx, int M, int K, int S, OzWorkspace& oz,
+                               cudaStream_t s) {
   const int Mp = ((M + TC_BM - 1) / TC_BM) * TC_BM, Kp = ((K + OZ_BK - 1) / OZ_BK) * OZ_BK;
   if (S > a.S_max || S < 1 || M <= 0 || K <= 0 || Mp > a.Mp_max ||
       (int64_t)3 * S * Mp * Kp > (int64_t)a.S_max * a.Mp_max * a.Kp_max)
     return cudaErrorInvalidValue;
   a.S = S; a.M = M; a.K = K; a.Mp = Mp; a.Kp = Kp; a.nz = 3;
   a.slice = (int64_t)Mp * Kp;
-  const int64_t zstride = (int64_t)S * a.slice;
-  if (op == OPC) {
-    oz_slice_hermitian3_kernel<<<M, 256, 0, s>>>(X, ldx, K, S, a.ptr, a.slice, zstride, Kp, Mp, a.e);
-    CHFSI_COUNT_LAUNCH();
-    return cudaGetLastError();
-  }
-  const int groups = (M + 31) / 32, kchunks = (K + 31) / 32;
-  oz_row_exponents3_kernel<<<groups, 256, 0, s>>>(X, ldx, M, K, 0, a.e, Mp);
-  CHFSI_COUNT_LAUNCH();
-  const int gy = std::max(1, std::min(kchunks, (4 * sm_count() + groups - 1) / groups));
-  const int chunk = 32 * ((kchunks + gy - 1) / gy);
-  oz_slice_rows3_kernel<<<dim3(groups, (K + chunk - 1) / chunk), 256, 0, s>>>(
-      X, ldx, M, K, S, 0, a.ptr, a.slice, zstride, Kp, a.e, Mp, chunk);
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  return slice_a_into(a, FORM_GAUSS, op, X, ldx, M, K, S, oz, s);
 }
 
-// op(B) (K x N) as the Gauss-form B operand, K-padding as the A operand's: op = OPN: column j
-// of X (optionally its lower half, as oz_slice_cols_kernel); op = OPC: the conjugated row j of
-// X (N x K).
-static cudaError_t oz_slice_b3(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, int S, int Kp,
-                               cudaStream_t s, int lower_half) {
+static cudaError_t oz_slice_b3(OzB& b, int op, const zd* X, int64_t ldx, int K, int N, int S, int Kp, OzWorkspace& oz,
+                               cudaStream_t s, int lower_half, const unsigned* key = nullptr,
+                               unsigned* clear = nullptr) {
   const int Np = oz_padded_n(N);
   if (S > b.S_max || S < 1 || N <= 0 || K <= 0 || Np > b.Np_max ||
       (int64_t)3 * S * Np * Kp > b.elems)
     return cudaErrorInvalidValue;
   b.S = S; b.N = N; b.Np = Np; b.Kp = Kp; b.nz = 3;
   b.slice = (int64_t)Np * Kp;
-  const int64_t zstride = (int64_t)S * b.slice;
-  if (op == OPC) {
-    const int groups = (N + 31) / 32, kchunks = (K + 31) / 32;
-    oz_row_exponents3_kernel<<<groups, 256, 0, s>>>(X, ldx, N, K, 1, b.e, Np);
-    CHFSI_COUNT_LAUNCH();
-    const int gy = std::max(1, std::min(kchunks, (4 * sm_count() + groups - 1) / groups));
-    const int chunk = 32 * ((kchunks + gy - 1) / gy);
-    oz_slice_rows3_kernel<<<dim3(groups, (K + chunk - 1) / chunk), 256, 0, s>>>(
-        X, ldx, N, K, S, 1, b.ptr, b.slice, zstride, Kp, b.e, Np, chunk);
-    CHFSI_COUNT_LAUNCH();
-    return cudaGetLastError();
-  }
-  oz_slice_cols3_kernel<<<N, 256, 0, s>>>(X, ldx, K, S, b.ptr, b.slice, zstride, Kp, Np, b.e, lower_half);
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  return slice_b_into(b, FORM_GAUSS, op, X, ldx, K, N, S, lower_half, oz, s, key, clear);
 }
 
 // ---- the Hermitian matrix of the filter (its slices stay in oz.H for the whole problem)
 cudaError_t oz_slice_hermitian(const zd* Hs, int64_t ldh, int n, int S, OzWorkspace& oz,
                                cudaStream_t s) {
-  if (oz_gauss(oz)) return oz_slice_a3(oz.H, OPC, Hs, ldh, n, n, S, s);
-  return oz_slice_a(oz.H, OPC, Hs, ldh, n, n, S, s);
+  if (oz_gauss(oz)) return oz_slice_a3(oz.H, OPC, Hs, ldh, n, n, S, oz, s);
+  return oz_slice_a(oz.H, OPC, Hs, ldh, n, n, S, oz, s);
 }
 
 // out(n x m) = alpha Hs Y + beta Cin + gamma D with Hs given by its slices in oz.H and Y
-// sliced here into S slices.
+// sliced here into S slices.  In a chain of products whose Y is the previous one's out (or its
+// first columns), keys_out of one and keys_in of the next hand the columns' scales on: the epilogue
+// that writes a block also finds them, which saves the next product a pass over it.
 cudaError_t oz_filter_product(const zd* Y, int64_t ldy, int n, int m, int S, double alpha,
                               double beta, const zd* Cin, int64_t ldcin, double gamma, const zd* D,
                               int64_t ldd, zd* out, int64_t ldo, OzWorkspace& oz, cudaStream_t s,
-                              cudaEvent_t ev_gemm_begin, cudaEvent_t ev_gemm_end) {
+                              cudaEvent_t ev_gemm_begin, cudaEvent_t ev_gemm_end, bool keys_in, bool keys_out) {
   if (m <= 0) return cudaSuccess;
   if (S > oz.H.S || S < 1 || oz.H.M != n) return cudaErrorInvalidValue;
-  cudaError_t e = oz.H.nz == 3 ? oz_slice_b3(oz.B, OPN, Y, ldy, n, m, S, oz.H.Kp, s, 0)
-                               : oz_slice_b(oz.B, OPN, Y, ldy, n, m, S, oz.H.Kp, s);
+  if (!oz_use_tcgen05()) keys_in = keys_out = false;
+  // keys of Y in buffer key_cur; the slicing clears the other buffer for the epilogue.  The keys'
+  // stride is the padded width of the product that left them: one of another width scans Y again
+  unsigned* clear = nullptr;
+  const unsigned* key = nullptr;
+  if (keys_in && oz.key_np == oz_padded_n(m)) key = oz.key[oz.key_cur];
+  if (keys_out) {
+    clear = oz.key[1 - oz.key_cur];
+    if (!key) CK_OZ(cudaMemsetAsync(clear, 0, sizeof(unsigned) * 3 * (size_t)oz_padded_n(m), s));
+  }
+  cudaError_t e = oz.H.nz == 3 ? oz_slice_b3(oz.B, OPN, Y, ldy, n, m, S, oz.H.Kp, oz, s, 0, key, key ? clear : nullptr)
+                               : oz_slice_b(oz.B, OPN, Y, ldy, n, m, S, oz.H.Kp, oz, s, 0, key, key ? clear : nullptr);
   if (e != cudaSuccess) return e;
-  return oz_product(oz.H, oz.B, S, alpha, beta, Cin, ldcin, gamma, D, ldd, out, ldo, 0, 0, oz, s,
-                    ev_gemm_begin, ev_gemm_end);
+  e = oz_product(oz.H, oz.B, S, alpha, beta, Cin, ldcin, gamma, D, ldd, out, ldo, 0, 0, oz, s,
+                 ev_gemm_begin, ev_gemm_end, 0, clear);
+  if (keys_out) {
+    oz.key_cur = 1 - oz.key_cur;
+    oz.key_np = oz_padded_n(m);
+  }
+  return e;
 }
 
 // General product with split operands: C = alpha op(A) op(B) + beta Cin + gamma D,
@@ -1608,11 +1616,9 @@ cudaError_t oz_gemm(int opA, const zd* A, int64_t lda, int opB, const zd* B, int
                     const zd* D, int64_t ldd, zd* C, int64_t ldc, int a_lower, int c_lower,
                     OzWorkspace& oz, cudaStream_t s, int b_tri, int b_lower_half) {
   const bool g3 = oz_gauss(oz);
-  cudaError_t e = g3 ? oz_slice_a3(oz.X, opA, A, lda, M, K, S, s) : oz_slice_a(oz.X, opA, A, lda, M, K, S, s);
-  if (e != cudaSuccess) return e;
-  e = g3 ? oz_slice_b3(oz.B, opB, B, ldb, K, N, S, oz.X.Kp, s, b_lower_half)
-         : oz_slice_b(oz.B, opB, B, ldb, K, N, S, oz.X.Kp, s, b_lower_half);
-  if (e != cudaSuccess) return e;
+  CK_OZ(g3 ? oz_slice_a3(oz.X, opA, A, lda, M, K, S, oz, s) : oz_slice_a(oz.X, opA, A, lda, M, K, S, oz, s));
+  CK_OZ(g3 ? oz_slice_b3(oz.B, opB, B, ldb, K, N, S, oz.X.Kp, oz, s, b_lower_half)
+           : oz_slice_b(oz.B, opB, B, ldb, K, N, S, oz.X.Kp, oz, s, b_lower_half));
   return oz_product(oz.X, oz.B, S, alpha, beta, Cin, ldcin, gamma, D, ldd, C, ldc, a_lower, c_lower, oz,
                     s, nullptr, nullptr, b_tri);
 }
@@ -1648,6 +1654,10 @@ cudaError_t oz_alloc(OzWorkspace& oz, int n_max, int blk_max, int S_max) {
   if (e != cudaSuccess) return e;
   e = cudaMalloc((void**)&oz.B.e, sizeof(int) * (size_t)3 * oz.B.Np_max);
   if (e != cudaSuccess) return e;
+  for (int k = 0; k < 2; ++k) {
+    e = cudaMalloc((void**)&oz.key[k], sizeof(unsigned) * (size_t)3 * std::max(oz.B.Np_max, oz.H.Mp_max));
+    if (e != cudaSuccess) return e;
+  }
   const int np_blk = ((blk_max + OZ_BN - 1) / OZ_BN) * OZ_BN;
   const size_t mp = (size_t)oz_padded_m(n_max);
   const size_t mp1 = (size_t)((n_max + TC_BM - 1) / TC_BM) * TC_BM;  // rows of a Gauss-form product
@@ -1658,7 +1668,8 @@ cudaError_t oz_alloc(OzWorkspace& oz, int n_max, int blk_max, int S_max) {
 }
 
 void oz_free(OzWorkspace& oz) {
-  void* ptrs[] = {oz.H.ptr, oz.H.e, oz.X.ptr, oz.X.e, oz.B.ptr, oz.B.e, oz.part};
+  void* ptrs[] = {oz.H.ptr, oz.H.e, oz.X.ptr, oz.X.e, oz.B.ptr, oz.B.e, oz.part,
+                  oz.key[0], oz.key[1]};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   oz = OzWorkspace{};
