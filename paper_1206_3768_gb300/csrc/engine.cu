@@ -388,7 +388,7 @@ int lanczos_run(chfsi_ctx* ctx, const zd* H, int64_t ldh, int n, int k, const zd
       return CHFSI_OK;
     }
   if (!ctx->capture_stream) CK(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
-  CK(hemv_rows_prepare(n, nullptr));
+  CK(hemv_rows_prepare(n));
   cudaGraph_t graph = nullptr;
   const long long before = g_kernel_launches;
   cudaError_t e = cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal);
@@ -427,14 +427,19 @@ int lanczos_issue(chfsi_ctx* ctx, cudaStream_t st, const zd* H, int64_t ldh, int
   CK(vec_norm(ws.lw, n, nrm, st));
   CK(vec_scale_into(ws.lw, n, nrm, V, st));
   for (int j = 0; j < k; ++j) {
-    CK(hemv_rows(H, ldh, V + (int64_t)j * ldv, ws.lw, n, st, ctx->opts.precision == 1));
+    if (ctx->opts.precision == 1)  // the first step leaves the narrowed matrix in the product scratch
+      CK(hemv_rows_f32(H, ldh, k > 1 ? reinterpret_cast<float2*>(ws.T) : nullptr, ws.n_max, j > 0,
+                       V + (int64_t)j * ldv, ws.lw, n, st));
+    else
+      CK(hemv_rows(H, ldh, V + (int64_t)j * ldv, ws.lw, n, st));
+    // two Gram-Schmidt passes, the second one's pieces of ||w||^2 in ws.lv
+    zd* c2 = ws.lc + lanczos_dot_parts() * (ws.lanczos_kmax + 1);
+    double* norm2 = reinterpret_cast<double*>(ws.lv);
     CK(block_dots(V, ldv, j, ws.lw, n, ws.lc, st));
-    CK(block_update(V, ldv, j, ws.lc, ws.lw, n, st));
-    CK(block_dots(V, ldv, j, ws.lw, n, ws.lc + (ws.lanczos_kmax + 1), st));
-    CK(block_update(V, ldv, j, ws.lc + (ws.lanczos_kmax + 1), ws.lw, n, st));
-    CK(vec_norm(ws.lw, n, nrm, st));
-    CK(lanczos_record(ws.lc, j, nrm, ws.lal, ws.lbe, st));
-    if (j + 1 < k) CK(vec_scale_into(ws.lw, n, nrm, V + (int64_t)(j + 1) * ldv, st));
+    CK(block_update(V, ldv, j, ws.lc, ws.lw, n, nullptr, st));
+    CK(block_dots(V, ldv, j, ws.lw, n, c2, st));
+    CK(block_update(V, ldv, j, c2, ws.lw, n, norm2, st));
+    CK(lanczos_next(ws.lw, n, norm2, ws.lc, j, ws.lal, ws.lbe, j + 1 < k ? V + (int64_t)(j + 1) * ldv : nullptr, st));
   }
   CK(tridiag_extremes(ws.lal, ws.lbe, k, out3, st));
   return CHFSI_OK;
@@ -1159,7 +1164,7 @@ cudaError_t workspace_alloc(Workspace& ws, int64_t n_max, int blk_max, int lancz
   AL(ws.Y0, nb); AL(ws.Y1, nb); AL(ws.F, nb); AL(ws.W, nb); AL(ws.YL, nb); AL(ws.Xw, nb); AL(ws.Z, nb);
   AL(ws.G, mm); AL(ws.V, mm); AL(ws.Rt, mm); AL(ws.jac, 3 * mp * mp);
   AL(ws.lv, n_max); AL(ws.lw, n_max); AL(ws.lV, n_max * (lanczos_kmax + 1));
-  AL(ws.lc, 2 * (lanczos_kmax + 1));
+  AL(ws.lc, 2 * lanczos_dot_parts() * (lanczos_kmax + 1));
   AL(ws.theta, ws.blk_max); AL(ws.theta2, ws.blk_max); AL(ws.resid, ws.blk_max);
   AL(ws.resid2, ws.blk_max); AL(ws.lamL, ws.blk_max); AL(ws.residL, ws.blk_max);
   AL(ws.gres, ws.blk_max); AL(ws.dscale, ws.blk_max); AL(ws.scal, 64);

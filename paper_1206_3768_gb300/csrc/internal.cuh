@@ -180,20 +180,28 @@ cudaError_t lock_scan(const double* r, int m, double tau, int max_lock, int* nlo
 cudaError_t fill_nan(double* x, int m, cudaStream_t s);
 
 // Lanczos pieces
-// w = H v for Hermitian H (row i read as column i); f32: FP32 multiply-adds (bound estimates).
-cudaError_t hemv_rows(const zd* H, int64_t ldh, const zd* v, zd* w, int n, cudaStream_t s, bool f32 = false);
-// Host-side set-up of the FP32 product for size n (kernel attribute, CTAs per SM with v in
-// shared memory; 0 when v stays in global memory), cached per host thread: called before a
-// stream capture so that none of it happens inside one.
-cudaError_t hemv_rows_prepare(int n, int* per_sm);
+// w = H v for Hermitian H (row i read as column i).
+cudaError_t hemv_rows(const zd* H, int64_t ldh, const zd* v, zd* w, int n, cudaStream_t s);
+// The same with FP32 multiply-adds (bound estimates).  copy (n x n float2, leading dimension ldc, or
+// nullptr): receives the narrowed matrix, or holds it already (have_copy) and is read instead.
+cudaError_t hemv_rows_f32(const zd* H, int64_t ldh, float2* copy, int64_t ldc, bool have_copy, const zd* v, zd* w,
+                          int n, cudaStream_t s);
+// Host-side set-up of the FP32 product for size n (kernel attributes, CTAs per SM with v in
+// shared memory), cached per host thread: called before a stream capture so that none of it
+// happens inside one.
+cudaError_t hemv_rows_prepare(int n);
+// c (lanczos_dot_parts() pieces per vector) = V_l^H w, l = 0..j; w -= V c, norm2 (optional, one per 64
+// rows): pieces of the new ||w||^2; then beta_j, alpha_j (from the first pass's c) and dst = w / beta_j
+// (or nullptr).
+int lanczos_dot_parts();
 cudaError_t block_dots(const zd* V, int64_t ldv, int j, const zd* w, int n, zd* c,
                        cudaStream_t s);
-cudaError_t block_update(const zd* V, int64_t ldv, int j, const zd* c, zd* w, int n,
+cudaError_t block_update(const zd* V, int64_t ldv, int j, const zd* c, zd* w, int n, double* norm2,
                          cudaStream_t s);
+cudaError_t lanczos_next(const zd* w, int n, const double* norm2, const zd* c, int j, double* alpha,
+                         double* beta, zd* dst, cudaStream_t s);
 cudaError_t vec_norm(const zd* w, int n, double* out, cudaStream_t s);
 cudaError_t vec_scale_into(const zd* w, int n, const double* nrm, zd* dst, cudaStream_t s);
-cudaError_t lanczos_record(const zd* c, int j, const double* nrm, double* alpha, double* beta,
-                           cudaStream_t s);
 cudaError_t tridiag_extremes(const double* alpha, const double* beta, int k, double* out3,
                              cudaStream_t s);
 

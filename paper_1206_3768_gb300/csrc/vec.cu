@@ -484,7 +484,16 @@ __device__ __forceinline__ float f32_trunc(double x) {
 // at most 8 terms, then FP64): relative error ~1e-7, enough for a spectral bound.  The
 // operands are narrowed by f32_trunc; v once per CTA into shared memory (vsh, n entries,
 // when the launch gives it room) or per use from global memory.
-__global__ void hemv_rows_f32_kernel(const zd* H, int64_t ldh, const zd* v, zd* w, int n, int v_in_smem) {
+// It is a stream of the matrix: what bounds it is the bytes in flight, so a lane loads its 8 (or
+// 16) entries of a block before it uses the first, and the first step of a run writes the narrowed
+// matrix (half the bytes) for the later ones to read; the sums are the same either way.
+// Measured, a run of 40 steps at n = 9300 with the vector kernels below: 27.8 -> 6.6 ms (545 us a product
+// before, 2.5 TB/s).
+enum { HEMV_F64 = 0, HEMV_F64_COPY = 1, HEMV_F32 = 2 };
+constexpr int HEMV_THREADS = 512;
+template <int MODE>
+__global__ void __launch_bounds__(HEMV_THREADS)
+    hemv_rows_f32_kernel(const zd* H, int64_t ldh, float2* C, int64_t ldc, const zd* v, zd* w, int n, int v_in_smem) {
   extern __shared__ float2 vsh[];
   const int lane = threadIdx.x & 31;
   const int warps = (blockDim.x >> 5) * gridDim.x;
@@ -497,14 +506,37 @@ __global__ void hemv_rows_f32_kernel(const zd* H, int64_t ldh, const zd* v, zd* 
   }
   for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
     const zd* col = H + (int64_t)i * ldh;
+    float2* cc = C + (int64_t)i * ldc;
     double sr = 0.0, si = 0.0;
-    for (int j0 = 0; j0 < n; j0 += 256) {
+    // entries j0 + 32 u + lane, u < 8, into h; past the end zeros (they add nothing to the sums)
+    auto load = [&](int j0, bool full, float2* h) {
+      if (MODE == HEMV_F32) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = j0 + u * 32 + lane;
+          h[u] = full || j < n ? cc[j] : make_float2(0.f, 0.f);
+        }
+      } else {
+        zd g[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = j0 + u * 32 + lane;
+          g[u] = full || j < n ? col[j] : zmk(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = j0 + u * 32 + lane;
+          h[u] = make_float2(f32_trunc(g[u].x), f32_trunc(g[u].y));
+          if (MODE == HEMV_F64_COPY && (full || j < n)) cc[j] = h[u];
+        }
+      }
+    };
+    auto add = [&](int j0, bool full, const float2* h) {
       float fr = 0.f, fi = 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int j = j0 + u * 32 + lane;
-        if (j < n) {
-          const zd h = col[j];
+        if (full || j < n) {
           float2 x;
           if (v_in_smem) {
             x = vsh[j];
@@ -512,13 +544,31 @@ __global__ void hemv_rows_f32_kernel(const zd* H, int64_t ldh, const zd* v, zd* 
             const zd xv = v[j];
             x = make_float2(f32_trunc(xv.x), f32_trunc(xv.y));
           }
-          const float hx = f32_trunc(h.x), hy = f32_trunc(h.y);
-          fr = fmaf(hx, x.x, fmaf(hy, x.y, fr));
-          fi = fmaf(hx, x.y, fmaf(-hy, x.x, fi));
+          fr = fmaf(h[u].x, x.x, fmaf(h[u].y, x.y, fr));
+          fi = fmaf(h[u].x, x.y, fmaf(-h[u].y, x.x, fi));
         }
       }
       sr += (double)fr;
       si += (double)fi;
+    };
+    int j0 = 0;
+    if (MODE == HEMV_F32)
+      for (; j0 + 512 <= n; j0 += 512) {
+        float2 h[16];
+        load(j0, true, h);
+        load(j0 + 256, true, h + 8);
+        add(j0, true, h);
+        add(j0 + 256, true, h + 8);
+      }
+    for (; j0 + 256 <= n; j0 += 256) {
+      float2 h[8];
+      load(j0, true, h);
+      add(j0, true, h);
+    }
+    if (j0 < n) {
+      float2 h[8];
+      load(j0, false, h);
+      add(j0, false, h);
     }
     sr = warp_sum(sr);
     si = warp_sum(si);
@@ -526,31 +576,80 @@ __global__ void hemv_rows_f32_kernel(const zd* H, int64_t ldh, const zd* v, zd* 
   }
 }
 
-// c_l = V_l^H w for l = 0..j  (one CTA per l)
+// One step's Gram-Schmidt pass against V (n x (j + 1)).  What bounds these kernels is FP64 latency (64
+// clocks an instruction of a warp) and how many SMs take part, so each dot product is shared by
+// DOT_PARTS CTAs, a row of the update by four lanes, and the pieces (few and in a fixed order) are
+// added where they are read.
+constexpr int DOT_PARTS = 4, UPD_ROWS = 64;
+
+// c[l * DOT_PARTS + q] = part q of V_l^H w, l = 0..j.  Grid: (j + 1, DOT_PARTS).
 __global__ void block_dots_kernel(const zd* V, int64_t ldv, const zd* w, int n, zd* c) {
-  const int l = blockIdx.x;
+  const int l = blockIdx.x, q = blockIdx.y, per = (n + DOT_PARTS - 1) / DOT_PARTS;
+  const int i1 = min(n, (q + 1) * per);
   double sr = 0.0, si = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = q * per + threadIdx.x; i < i1; i += blockDim.x) {
     const zd a = V[i + (int64_t)l * ldv], b = w[i];
-    sr += a.x * b.x + a.y * b.y;
-    si += a.x * b.y - a.y * b.x;
+    sr = fma(a.x, b.x, fma(a.y, b.y, sr));
+    si = fma(a.x, b.y, fma(-a.y, b.x, si));
   }
   sr = block_sum(sr);
   si = block_sum(si);
-  if (threadIdx.x == 0) c[l] = zmk(sr, si);
+  if (threadIdx.x == 0) c[l * DOT_PARTS + q] = zmk(sr, si);
 }
 
-// w -= V c  (V: n x (j+1))
-__global__ void block_update_kernel(const zd* V, int64_t ldv, int jp1, const zd* c, zd* w, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    zd s = w[i];
-    for (int l = 0; l < jp1; ++l) {
-      const zd a = V[i + (int64_t)l * ldv], cl = c[l];
-      s.x -= a.x * cl.x - a.y * cl.y;
-      s.y -= a.x * cl.y + a.y * cl.x;
-    }
-    w[i] = s;
+__device__ __forceinline__ zd dot_total(const zd* c, int l) {
+  zd s = c[l * DOT_PARTS];
+#pragma unroll
+  for (int q = 1; q < DOT_PARTS; ++q) s = zadd(s, c[l * DOT_PARTS + q]);
+  return s;
+}
+
+// w -= V c; norm2 (optional): sum of |w_i|^2 over the CTA's rows.  UPD_ROWS rows a CTA, four lanes each.
+__global__ void __launch_bounds__(4 * UPD_ROWS)
+    block_update_kernel(const zd* V, int64_t ldv, int jp1, const zd* c, zd* w, int n, double* norm2) {
+  extern __shared__ zd cs[];
+  for (int l = threadIdx.x; l < jp1; l += blockDim.x) cs[l] = dot_total(c, l);
+  __syncthreads();
+  const int i = blockIdx.x * UPD_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
+  zd s = zmk(0.0, 0.0);
+  if (i < n) {
+#pragma unroll 4
+    for (int l = q; l < jp1; l += 4) s = zfma(V[i + (int64_t)l * ldv], cs[l], s);
   }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  double v2 = 0.0;
+  if (i < n && q == 0) {
+    const zd r = zsub(w[i], s);
+    w[i] = r;
+    v2 = zabs2(r);
+  }
+  if (norm2) {
+    v2 = block_sum(v2);
+    if (threadIdx.x == 0) norm2[blockIdx.x] = v2;
+  }
+}
+
+// End of step j: beta_j = ||w|| from the update's pieces, alpha_j = Re c_j of the first pass, and
+// (dst) the next basis vector w / beta_j.
+__global__ void lanczos_next_kernel(const zd* w, int n, const double* norm2, int parts, const zd* c, int j,
+                                    double* alpha, double* beta, zd* dst) {
+  double s = 0.0;
+  for (int i = threadIdx.x; i < parts; i += blockDim.x) s += norm2[i];
+  s = block_sum(s);
+  __shared__ double nrm;
+  if (threadIdx.x == 0) nrm = sqrt(s);
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    alpha[j] = dot_total(c, j).x;
+    beta[j] = nrm;
+  }
+  if (!dst) return;
+  const double inv = 1.0 / nrm;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = zscale(w[i], inv);
 }
 
 __global__ void vec_norm_kernel(const zd* w, int n, double* out) {
@@ -566,56 +665,90 @@ __global__ void vec_scale_into_kernel(const zd* w, int n, const double* nrm, zd*
     dst[i] = zscale(w[i], inv);
 }
 
-__global__ void lanczos_record_kernel(const zd* c, int j, const double* nrm, double* alpha,
-                                      double* beta) {
-  if (threadIdx.x == 0) {
-    alpha[j] = c[j].x;
-    beta[j] = nrm[0];
-  }
-}
-
-// Number of eigenvalues of the symmetric tridiagonal T (alpha, beta) below x (Sturm).
-__device__ int sturm_count(const double* al, const double* be, int k, double x) {
+// Number of eigenvalues below x of the symmetric tridiagonal T (diagonal al, squared off-diagonal
+// b2, entries of order 1 at most): sign changes of the leading minors p_i = (al_i - x) p_{i-1} -
+// b2_{i-1} p_{i-2}.  A zero minor keeps the sign before it.  The pair is rescaled by a power of two
+// when it leaves the middle of the range (checked every step on the exponents; a step shrinks it
+// by at most b2).  Three FP64 instructions a step, where the quotients q_i = p_i / p_{i-1} take a
+// division of 1442 clocks.
+__device__ int sturm_count(const double* al, const double* b2, int k, double x) {
   int cnt = 0;
-  double q = al[0] - x;
-  if (q < 0.0) ++cnt;
+  bool neg = false;
+  double p2 = 1.0, p1 = al[0] - x;
+  if (p1 < 0.0) { cnt = 1; neg = true; }
   for (int i = 1; i < k; ++i) {
-    if (q == 0.0) q = 1e-300;
-    q = (al[i] - x) - be[i - 1] * be[i - 1] / q;
-    if (q < 0.0) ++cnt;
+    const double p = fma(al[i] - x, p1, -b2[i - 1] * p2);
+    p2 = p1;
+    p1 = p;
+    if (neg ? p > 0.0 : p < 0.0) { neg = !neg; ++cnt; }  // (not a number: no change)
+    const int e = max((__double2hiint(p1) >> 20) & 0x7FF, (__double2hiint(p2) >> 20) & 0x7FF);
+    if (e < 1023 - 300 || e > 1023 + 300) {
+      const double f = e < 1023 ? 0x1p300 : 0x1p-300;
+      p1 *= f;
+      p2 *= f;
+    }
   }
   return cnt;
 }
 
-// out[0] = min eig(T_k), out[1] = max eig(T_k), out[2] = max eig + |beta_{k-1}|.
-__global__ void tridiag_extremes_kernel(const double* al, const double* be, int k, double* out) {
-  if (threadIdx.x != 0) return;
-  double lo = al[0], hi = al[0];
-  for (int i = 0; i < k; ++i) {
+// out[0] = min eig(T_k), out[1] = max eig(T_k), out[2] = max eig + |beta_{k-1}|: warp 0 looks for the
+// smallest, warp 1 for the largest eigenvalue, 32 points of the interval at a time (an interval
+// shrinks by 33 a round, to neighbouring doubles in about 11; one thread bisecting with divisions
+// took 1.1 ms at k = 20 and 2.2 ms at k = 40).  T is scaled by a power of two to a bound in [1/2, 1).
+__global__ void __launch_bounds__(64) tridiag_extremes_kernel(const double* al, const double* be, int k, double* out) {
+  extern __shared__ double tri[];  // k: scaled diagonal; k: scaled squared off-diagonal
+  __shared__ double ext[2];
+  const int tid = threadIdx.x, lane = tid & 31;
+  double lo = INFINITY, hi = -INFINITY;
+  for (int i = lane; i < k; i += 32) {
     const double rad = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i < k - 1 ? fabs(be[i]) : 0.0);
     lo = fmin(lo, al[i] - rad);
     hi = fmax(hi, al[i] + rad);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  int shift = 0;
+  const double bound = fmax(fabs(lo), fabs(hi));
+  if (bound > 0.0 && isfinite(bound)) frexp(bound, &shift);
+  const double down = ldexp(1.0, -shift);
+  for (int i = tid; i < k; i += 64) {
+    const double b = i < k - 1 ? be[i] * down : 0.0;
+    tri[i] = al[i] * down;
+    tri[k + i] = b * b;
+  }
+  lo *= down;
+  hi *= down;
   const double pad = 1e-12 * fmax(fabs(lo), fabs(hi)) + 1e-300;
-  lo -= pad;
-  hi += pad;
-  // smallest: largest x with count(x) == 0
-  double a = lo, b = hi;
-  for (int it = 0; it < 200 && b - a > 0.0; ++it) {
-    const double mid = 0.5 * (a + b);
-    if (mid <= a || mid >= b) break;
-    if (sturm_count(al, be, k, mid) >= 1) b = mid; else a = mid;
+  __syncthreads();
+  // smallest: count reaches 1; largest: count reaches k
+  const int want = tid < 32 ? 1 : k;
+  double a = lo - pad, b = hi + pad;
+  for (int round = 0; round < 40 && b > a; ++round) {
+    const double x = fma((b - a) * (1.0 / 33.0), (double)(lane + 1), a);
+    const bool inside = x > a && x < b;
+    const unsigned at = __ballot_sync(0xffffffffu, inside && sturm_count(tri, tri + k, k, x) >= want);
+    const unsigned in = __ballot_sync(0xffffffffu, inside);
+    if (in == 0u) break;  // no double between a and b
+    const unsigned below = in & ~at;  // points inside that do not reach it
+    const int first = at ? __ffs(at) - 1 : -1;
+    // the last point below the first that reaches it
+    const unsigned before = first >= 0 ? below & ((1u << first) - 1u) : below;
+    const double na = before ? __shfl_sync(0xffffffffu, x, 31 - __clz(before)) : a;
+    const double nb = first >= 0 ? __shfl_sync(0xffffffffu, x, first) : b;
+    if (na == a && nb == b) break;
+    a = na;
+    b = nb;
   }
-  out[0] = 0.5 * (a + b);
-  // largest: smallest x with count(x) == k
-  a = lo; b = hi;
-  for (int it = 0; it < 200 && b - a > 0.0; ++it) {
-    const double mid = 0.5 * (a + b);
-    if (mid <= a || mid >= b) break;
-    if (sturm_count(al, be, k, mid) >= k) b = mid; else a = mid;
+  if (lane == 0) ext[tid >> 5] = ldexp(0.5 * (a + b), shift);
+  __syncthreads();
+  if (tid == 0) {
+    out[0] = ext[0];
+    out[1] = ext[1];
+    out[2] = ext[1] + fabs(be[k - 1]);
   }
-  out[1] = 0.5 * (a + b);
-  out[2] = out[1] + fabs(be[k - 1]);
 }
 
 inline int grid_for(int64_t total, int threads = 256) {
@@ -856,50 +989,92 @@ cudaError_t fill_nan(double* x, int m, cudaStream_t s) {
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
-cudaError_t hemv_rows_prepare(int n, int* per_sm) {
+// CTAs per SM of the three forms with v in shared memory (0: v stays in global memory).
+static const void* hemv_f32_kernel(int mode) {
+  return mode == HEMV_F32        ? (const void*)hemv_rows_f32_kernel<HEMV_F32>
+         : mode == HEMV_F64_COPY ? (const void*)hemv_rows_f32_kernel<HEMV_F64_COPY>
+                                 : (const void*)hemv_rows_f32_kernel<HEMV_F64>;
+}
+static cudaError_t hemv_f32_occupancy(int n, int mode, int* per_sm) {
   constexpr size_t kVshMax = 128 * 1024;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      hemv_rows_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVshMax);
-  if (attr != cudaSuccess) return attr;
-  static thread_local int last_n = -1, last_per_sm = 0;
-  const size_t smem = sizeof(float2) * (size_t)n;
-  if (n != last_n) {
-    int p = 0;
-    if (n > 0 && smem <= kVshMax) {
-      const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, hemv_rows_f32_kernel, 256, smem);
+  static const cudaError_t attr = [] {
+    for (int m = 0; m < 3; ++m) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(hemv_f32_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVshMax);
       if (e != cudaSuccess) return e;
     }
-    last_n = n;
-    last_per_sm = p;
+    return cudaSuccess;
+  }();
+  if (attr != cudaSuccess) return attr;
+  static thread_local int last_n[3] = {-1, -1, -1}, last_per_sm[3] = {0, 0, 0};
+  const size_t smem = sizeof(float2) * (size_t)n;
+  if (n != last_n[mode]) {
+    int p = 0;
+    if (n > 0 && smem <= kVshMax) {
+      const cudaError_t e =
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, hemv_f32_kernel(mode), HEMV_THREADS, smem);
+      if (e != cudaSuccess) return e;
+    }
+    last_n[mode] = n;
+    last_per_sm[mode] = p;
   }
-  if (per_sm) *per_sm = last_per_sm;
+  *per_sm = last_per_sm[mode];
   return cudaSuccess;
 }
-cudaError_t hemv_rows(const zd* H, int64_t ldh, const zd* v, zd* w, int n, cudaStream_t s, bool f32) {
+cudaError_t hemv_rows_prepare(int n) {
+  int per_sm = 0;
+  cudaError_t e = cudaSuccess;
+  for (int m = 0; m < 3 && e == cudaSuccess; ++m) e = hemv_f32_occupancy(n, m, &per_sm);
+  return e;
+}
+cudaError_t hemv_rows(const zd* H, int64_t ldh, const zd* v, zd* w, int n, cudaStream_t s) {
   const int warps_per_block = 8;
-  int blocks = std::max(1, std::min((n + warps_per_block - 1) / warps_per_block, 16 * sm_count()));
-  if (f32) {
-    // v in shared memory up to 128 KB (n <= 16384), with as many CTAs as fit on the SMs
-    int per_sm = 0;
-    const cudaError_t e = hemv_rows_prepare(n, &per_sm);
-    if (e != cudaSuccess) return e;
-    const int in_smem = per_sm > 0 ? 1 : 0;
-    if (in_smem) blocks = std::max(1, std::min(blocks, per_sm * sm_count()));
-    hemv_rows_f32_kernel<<<blocks, 32 * warps_per_block, in_smem ? sizeof(float2) * (size_t)n : 0, s>>>(
-        H, ldh, v, w, n, in_smem);
-  } else {
-    hemv_rows_kernel<<<blocks, 32 * warps_per_block, 0, s>>>(H, ldh, v, w, n);
-  }
+  const int blocks = std::max(1, std::min((n + warps_per_block - 1) / warps_per_block, 16 * sm_count()));
+  hemv_rows_kernel<<<blocks, 32 * warps_per_block, 0, s>>>(H, ldh, v, w, n);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
+cudaError_t hemv_rows_f32(const zd* H, int64_t ldh, float2* copy, int64_t ldc, bool have_copy, const zd* v, zd* w,
+                          int n, cudaStream_t s) {
+  const int mode = have_copy ? HEMV_F32 : (copy ? HEMV_F64_COPY : HEMV_F64);
+  // v in shared memory up to 128 KB (n <= 16384), with as many CTAs as fit on the SMs
+  int per_sm = 0;
+  const cudaError_t e = hemv_f32_occupancy(n, mode, &per_sm);
+  if (e != cudaSuccess) return e;
+  const int in_smem = per_sm > 0 ? 1 : 0, rows = HEMV_THREADS / 32;
+  int blocks = std::max(1, std::min((n + rows - 1) / rows, 16 * sm_count()));
+  if (in_smem) blocks = std::max(1, std::min(blocks, per_sm * sm_count()));
+  const size_t smem = in_smem ? sizeof(float2) * (size_t)n : 0;
+  if (mode == HEMV_F32)
+    hemv_rows_f32_kernel<HEMV_F32><<<blocks, HEMV_THREADS, smem, s>>>(H, ldh, copy, ldc, v, w, n, in_smem);
+  else if (mode == HEMV_F64_COPY)
+    hemv_rows_f32_kernel<HEMV_F64_COPY><<<blocks, HEMV_THREADS, smem, s>>>(H, ldh, copy, ldc, v, w, n, in_smem);
+  else
+    hemv_rows_f32_kernel<HEMV_F64><<<blocks, HEMV_THREADS, smem, s>>>(H, ldh, copy, ldc, v, w, n, in_smem);
+  CHFSI_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+int lanczos_dot_parts() { return DOT_PARTS; }
 cudaError_t block_dots(const zd* V, int64_t ldv, int j, const zd* w, int n, zd* c, cudaStream_t s) {
-  block_dots_kernel<<<j + 1, 256, 0, s>>>(V, ldv, w, n, c);
+  block_dots_kernel<<<dim3(j + 1, DOT_PARTS), 256, 0, s>>>(V, ldv, w, n, c);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
-cudaError_t block_update(const zd* V, int64_t ldv, int j, const zd* c, zd* w, int n, cudaStream_t s) {
-  block_update_kernel<<<grid_for(n), 256, 0, s>>>(V, ldv, j + 1, c, w, n);
+cudaError_t block_update(const zd* V, int64_t ldv, int j, const zd* c, zd* w, int n, double* norm2, cudaStream_t s) {
+  const size_t smem = sizeof(zd) * (size_t)(j + 1);
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(block_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  block_update_kernel<<<(n + UPD_ROWS - 1) / UPD_ROWS, 4 * UPD_ROWS, smem, s>>>(V, ldv, j + 1, c, w, n, norm2);
+  CHFSI_COUNT_LAUNCH();
+  return cudaGetLastError();
+}
+cudaError_t lanczos_next(const zd* w, int n, const double* norm2, const zd* c, int j, double* alpha, double* beta,
+                         zd* dst, cudaStream_t s) {
+  lanczos_next_kernel<<<dst ? grid_for(n) : 1, 256, 0, s>>>(w, n, norm2, (n + UPD_ROWS - 1) / UPD_ROWS, c, j, alpha,
+                                                            beta, dst);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -913,15 +1088,15 @@ cudaError_t vec_scale_into(const zd* w, int n, const double* nrm, zd* dst, cudaS
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
-cudaError_t lanczos_record(const zd* c, int j, const double* nrm, double* alpha, double* beta,
-                           cudaStream_t s) {
-  lanczos_record_kernel<<<1, 32, 0, s>>>(c, j, nrm, alpha, beta);
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
-}
 cudaError_t tridiag_extremes(const double* alpha, const double* beta, int k, double* out3,
                              cudaStream_t s) {
-  tridiag_extremes_kernel<<<1, 32, 0, s>>>(alpha, beta, k, out3);
+  const size_t smem = 2 * sizeof(double) * (size_t)k;
+  if (smem > 48 * 1024) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(tridiag_extremes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  tridiag_extremes_kernel<<<1, 64, smem, s>>>(alpha, beta, k, out3);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
