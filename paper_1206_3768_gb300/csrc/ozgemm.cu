@@ -34,6 +34,17 @@
 
 namespace {
 
+// Programmatic dependent launch: a product is a chain of three or four short kernels, and the launch
+// latency between them is a good part of a small one.  Each of them lets its successor start as
+// soon as all its CTAs run (launch_dependents first) and waits for its own predecessor to have
+// finished, with all its writes, before it touches memory (wait; it returns at once in an ordinary
+// launch).  Since every kernel of the chain waits, the order of all reads and writes is that of
+// the stream.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
 constexpr int OZ_BM = 128, OZ_BN = 64, OZ_BK = 64, OZ_THREADS = 256, OZ_STAGES = 3;
 constexpr int OZ_BETA = 7;         // bits per digit slice
 constexpr int OZ_CHUNK_KB = 15;    // k-blocks of 64 per exact FP32 chunk (960 terms: 960 * 129^2 < 2^24)
@@ -619,6 +630,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
   tc_fence_before();
+  pdl_enter();  // set-up overlaps the end of the slicing; every thread waits before any copy or write
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
@@ -884,6 +896,7 @@ struct ColumnSource {
 // Keys of the columns' parts: key[part * stride + j], raised by atomicMax (cleared before).  Grid:
 // (row chunks, columns).
 __global__ void oz_col_keys_kernel(const ColumnSource src, int parts, unsigned* key, int stride, int chunk) {
+  pdl_enter();
   const int j = blockIdx.y, k1 = min(src.n, (int)(blockIdx.x + 1) * chunk);
   unsigned m0 = 0, m1 = 0, m2 = 0;
   for (int k = blockIdx.x * chunk + threadIdx.x; k < k1; k += blockDim.x) {
@@ -915,6 +928,7 @@ template <int FORM>
 __global__ void oz_slice_cols_kernel(const ColumnSource src, int S, __nv_bfloat16* out, int64_t slice,
                                      int64_t zstride, int Kp, int* e_out, int e_stride, const unsigned* key,
                                      unsigned* clear, int chunk) {
+  pdl_enter();
   constexpr int parts = FORM == FORM_GAUSS ? 3 : 1;
   const int j = blockIdx.y, tid = threadIdx.x;
   unsigned kz[3] = {0, 0, 0};
@@ -976,6 +990,7 @@ __global__ void oz_slice_cols_kernel(const ColumnSource src, int S, __nv_bfloat1
 // column (coalesced), the columns shared out over blockIdx.y.
 __global__ void oz_row_keys_kernel(const zd* X, int64_t ldx, int rows, int cols, int conj, int parts, unsigned* key,
                                    int stride) {
+  pdl_enter();
   __shared__ unsigned red[3][8][32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const int r = blockIdx.x * 32 + tx;
@@ -1006,6 +1021,7 @@ template <int FORM>
 __global__ void oz_slice_rows_kernel(const zd* X, int64_t ldx, int rows, int cols, int S, int conj,
                                      __nv_bfloat16* out, int64_t slice, int64_t zstride, int Kp, int* e_out,
                                      int e_stride, const unsigned* key, int chunk) {
+  pdl_enter();
   constexpr int parts = FORM == FORM_GAUSS ? 3 : 1;
   __shared__ int ex[3][32];
   __shared__ zd tile[32][33];
@@ -1070,19 +1086,21 @@ __device__ __forceinline__ double scaled_sum(float h, float l, int ex) {
 // i (P2 - P0 - P1) from the Gauss form's three products.  key (optional): the keys of the columns of
 // out, for the slices of the next product (cleared before).  Grid: (row chunks, columns).
 // What bounds it: 13 FP64 instructions an entry on large blocks (n = 9300, m = 320: 195 -> 113 us), the
-// chain of loads on small ones, which is why the splits' loads are issued in groups of four.
+// chain of loads on small ones, which is why the splits' loads are issued in groups.
+constexpr int EPI_THREADS = 128;
 template <int NZ>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(EPI_THREADS)
     oz_epilogue_kernel(const float2* part, int splits, int Mp, int Np, const int* eA, const int* eB, int n,
                        double alpha, double beta, const zd* Cin, int64_t ldcin, double gamma, const zd* D,
                        int64_t ldd, zd* out, int64_t ldo, int lower, unsigned* key, int key_stride, int rows) {
+  pdl_enter();
   const int64_t prod = (int64_t)Mp * Np, zst = splits * prod;
   const int i1 = min(n, (int)(blockIdx.x + 1) * rows), j = blockIdx.y;
   int eb[NZ];
 #pragma unroll
   for (int z = 0; z < NZ; ++z) eb[z] = eB[z * Np + j];
   unsigned m0 = 0, m1 = 0, m2 = 0;
-  for (int i = blockIdx.x * rows + threadIdx.x; i < i1; i += 256) {
+  for (int i = blockIdx.x * rows + threadIdx.x; i < i1; i += EPI_THREADS) {
     if (lower && j > i) continue;
     const zd cin = beta != 0.0 ? Cin[i + (int64_t)j * ldcin] : zmk(0.0, 0.0);
     const zd d = gamma != 0.0 ? D[i + (int64_t)j * ldd] : zmk(0.0, 0.0);
@@ -1104,7 +1122,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int z = 0; z < 3; ++z) {
         float h = 0.f, l = 0.f;
-#pragma unroll 4
+#pragma unroll 8
         for (int sp = 0; sp < splits; ++sp) {
           const float2 q = part[z * zst + sp * prod + (int64_t)j * Mp + i];
           two_sum_acc(h, l, q.x);
@@ -1261,6 +1279,25 @@ int oz_padded_n(int m) {
     if (e_ != cudaSuccess) return e_; \
   } while (0)
 
+// Launch with programmatic stream serialization (see pdl_enter; kernels that call it only).
+template <class... P, class... A>
+static cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s,
+                                  A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  if (e == cudaSuccess) CHFSI_COUNT_LAUNCH();
+  return e;
+}
+
 // Where a sliced operand goes: buffer, scales and layout.
 struct SliceDst {
   __nv_bfloat16* ptr;
@@ -1283,23 +1320,16 @@ static cudaError_t slice_cols(const ColumnSource& src, int cols, const SliceDst&
     if (!key) {
       const int parts = d.form == FORM_GAUSS ? 3 : 1;
       CK_OZ(cudaMemsetAsync(oz.key[oz.key_cur], 0, sizeof(unsigned) * (size_t)parts * d.e_stride, s));
-      oz_col_keys_kernel<<<dim3(gx, cols), 256, 0, s>>>(src, parts, oz.key[oz.key_cur], d.e_stride, chunk);
-      CHFSI_COUNT_LAUNCH();
+      CK_OZ(launch_chained(oz_col_keys_kernel, dim3(gx, cols), 256, 0, s, src, parts, oz.key[oz.key_cur], d.e_stride,
+                           chunk));
       key = oz.key[oz.key_cur];
     }
   }
-  const dim3 grid(gx, cols);
-  if (d.form == FORM_GAUSS)
-    oz_slice_cols_kernel<FORM_GAUSS><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e, d.e_stride,
-                                                          key, clear, chunk);
-  else if (d.form == FORM_EMBED_A)
-    oz_slice_cols_kernel<FORM_EMBED_A><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e,
-                                                            d.e_stride, key, clear, chunk);
-  else
-    oz_slice_cols_kernel<FORM_EMBED_B><<<grid, 256, 0, s>>>(src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e,
-                                                            d.e_stride, key, clear, chunk);
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  const auto kernel = d.form == FORM_GAUSS     ? oz_slice_cols_kernel<FORM_GAUSS>
+                      : d.form == FORM_EMBED_A ? oz_slice_cols_kernel<FORM_EMBED_A>
+                                               : oz_slice_cols_kernel<FORM_EMBED_B>;
+  return launch_chained(kernel, dim3(gx, cols), 256, 0, s, src, d.S, d.ptr, d.slice, d.zstride, d.Kp, d.e, d.e_stride,
+                        key, clear, chunk);
 }
 
 // Slices of the rows of X (rows x cols) or of its conjugate: keys, then digits by (32-row group, column
@@ -1310,21 +1340,14 @@ static cudaError_t slice_rows(const zd* X, int64_t ldx, int rows, int cols, int 
   unsigned* key = oz.key[oz.key_cur];
   CK_OZ(cudaMemsetAsync(key, 0, sizeof(unsigned) * (size_t)parts * d.e_stride, s));
   const int gy = std::max(1, std::min(kchunks, (4 * sm_count() + groups - 1) / groups));
-  oz_row_keys_kernel<<<dim3(groups, gy), 256, 0, s>>>(X, ldx, rows, cols, conj, parts, key, d.e_stride);
-  CHFSI_COUNT_LAUNCH();
+  CK_OZ(launch_chained(oz_row_keys_kernel, dim3(groups, gy), 256, 0, s, X, ldx, rows, cols, conj, parts, key,
+                       d.e_stride));
   const int chunk = 32 * ((kchunks + gy - 1) / gy);
-  const dim3 grid(groups, (cols + chunk - 1) / chunk);
-  if (d.form == FORM_GAUSS)
-    oz_slice_rows_kernel<FORM_GAUSS><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
-                                                          d.Kp, d.e, d.e_stride, key, chunk);
-  else if (d.form == FORM_EMBED_A)
-    oz_slice_rows_kernel<FORM_EMBED_A><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
-                                                            d.Kp, d.e, d.e_stride, key, chunk);
-  else
-    oz_slice_rows_kernel<FORM_EMBED_B><<<grid, 256, 0, s>>>(X, ldx, rows, cols, d.S, conj, d.ptr, d.slice, d.zstride,
-                                                            d.Kp, d.e, d.e_stride, key, chunk);
-  CHFSI_COUNT_LAUNCH();
-  return cudaGetLastError();
+  const auto kernel = d.form == FORM_GAUSS     ? oz_slice_rows_kernel<FORM_GAUSS>
+                      : d.form == FORM_EMBED_A ? oz_slice_rows_kernel<FORM_EMBED_A>
+                                               : oz_slice_rows_kernel<FORM_EMBED_B>;
+  return launch_chained(kernel, dim3(groups, (cols + chunk - 1) / chunk), 256, 0, s, X, ldx, rows, cols, d.S, conj,
+                        d.ptr, d.slice, d.zstride, d.Kp, d.e, d.e_stride, key, chunk);
 }
 
 // op(A) (M x K) as the A operand.  op = OPC: row i of op(A) is the conjugated column i of X (K x M,
@@ -1441,9 +1464,7 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     if (tc_attr != cudaSuccess) return tc_attr;
     auto launch = [&](int sp) -> cudaError_t {
       tp.splits = sp;
-      oz_gemm_tc_kernel<<<dim3(tiles, sp, nz), TC_THREADS, smem, s>>>(mapA, mapB, tp);
-      CHFSI_COUNT_LAUNCH();
-      return cudaGetLastError();
+      return launch_chained(oz_gemm_tc_kernel, dim3(tiles, sp, nz), TC_THREADS, smem, s, mapA, mapB, tp);
     };
     // split count: the wave model's choice, or the fastest of a few candidates around it,
     // measured on the first product of each shape and kept for the process (autotuner)
@@ -1519,16 +1540,12 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     oz_mma_epilogue_kernel<<<blocks, 256, 0, s>>>(oz.part, splits, Mp, Np, a.e, b.e, n, m, alpha, beta, Cin, ldcin,
                                                   gamma, D, ldd, out, ldo, c_lower);
   } else {
-    // 1024 rows a CTA of 256 threads, 256 while that leaves less than eight CTAs per SM
-    const int rows = (int64_t)((n + 1023) / 1024) * m >= 8 * sm_count() ? 1024 : 256;
+    // 1024 rows a CTA, 128 (one per thread) while that leaves less than eight CTAs per SM
+    const int rows = (int64_t)((n + 1023) / 1024) * m >= 8 * sm_count() ? 1024 : EPI_THREADS;
     const dim3 grid((n + rows - 1) / rows, m);
-    const float2* part = reinterpret_cast<const float2*>(oz.part);
-    if (nz == 3)
-      oz_epilogue_kernel<3><<<grid, 256, 0, s>>>(part, splits, Mp, Np, a.e, b.e, n, alpha, beta, Cin, ldcin, gamma, D,
-                                                 ldd, out, ldo, c_lower, key_out, Np, rows);
-    else
-      oz_epilogue_kernel<1><<<grid, 256, 0, s>>>(part, splits, Mp, Np, a.e, b.e, n, alpha, beta, Cin, ldcin, gamma, D,
-                                                 ldd, out, ldo, c_lower, key_out, Np, rows);
+    return launch_chained(nz == 3 ? oz_epilogue_kernel<3> : oz_epilogue_kernel<1>, grid, EPI_THREADS, 0, s,
+                          reinterpret_cast<const float2*>(oz.part), splits, Mp, Np, a.e, b.e, n, alpha, beta, Cin,
+                          ldcin, gamma, D, ldd, out, ldo, c_lower, key_out, Np, rows);
   }
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
