@@ -83,3 +83,18 @@ def test_fp64_product_tiles_and_splits(M, N, K, opa, opb):
     want = 0.7 * (a @ b) - 1.3 * C
     bound = 3 * (K + 4) * U * (2 * np.abs(a) @ np.abs(b) + np.abs(C))
     assert np.all(np.abs(got - want) <= bound)
+
+
+@pytest.mark.parametrize("M,N,K", [(427, 59, 427), (562, 12, 562), (700, 30, 1100)])
+def test_fp64_product_sums_in_short_pieces(M, N, K):
+    # Sums of K positive terms.  One after another their rounding errors add up to about U / 2 sqrt(K) / 3
+    # of the sum (3.4 U at K = 427, 5.5 U at 1100); in S pieces of at most 128 terms to U / 2
+    # (sqrt(128 / S) / 3 + sqrt(S) / 3), below 1.5 U for S = 4 .. 18.
+    rng = np.random.default_rng([M, N, K])
+    a, b = rng.uniform(0.5, 1.0, (M, K)), rng.uniform(0.5, 1.0, (K, N))
+    with cb.Solver(1100, 130, precision=0) as s:
+        got = cb.chfsi_zgemm(s.ctx, "N", "N", 1.0, torch.from_numpy(a.astype(complex)).cuda(),
+                             torch.from_numpy(b.astype(complex)).cuda(), 0.0,
+                             torch.zeros(M, N, dtype=torch.complex128).cuda()).cpu().numpy().real
+    want = np.matmul(a.astype(np.longdouble), b.astype(np.longdouble))
+    assert np.sqrt(np.mean(((got - want) / want) ** 2)) <= 1.5 * U
