@@ -619,7 +619,7 @@ int orthonormalize_block(chfsi_ctx* ctx, int n, int m, zd** Ya, zd** Yb, const z
 
 // Narrowest Rayleigh-Ritz block whose eigensolver runs in double-float arithmetic in mixed
 // precision: environment variable CHFSI_JACOBI_DF_MIN (default 512 columns; FP64 and double-float,
-// near-diagonal matrices: 11.6 and 16.2 ms at 383 columns, 17.2 and 18.9 at 450, 35.2 and 30.7 at 600).
+// near-diagonal matrices: 11.7 and 15.9 ms at 383 columns, 17.3 and 18.7 at 450, 23.9 and 21.8 at 512, 36.7 and 30.8 at 600).
 int jacobi_df_min() {
   static const int v = [] {
     const char* e = std::getenv("CHFSI_JACOBI_DF_MIN");

@@ -53,3 +53,18 @@ def test_heev_of_diagonal_and_zero_matrices():
                 w, V = (x.cpu().numpy() for x in cb.chfsi_heev(s.ctx, torch.from_numpy(A).cuda()))
                 assert np.array_equal(w, np.sort(A.diagonal().real))
                 assert np.array_equal(np.abs(V).sum(0), np.ones(m)) and np.array_equal(A @ V, V * w)
+
+
+@pytest.mark.parametrize("m", [15, 37, 64, 97, 217])
+def test_heev_leaves_no_more_than_its_threshold(m):
+    # close eigenvalues turn what is left off the diagonal of V^H A V into eigenvector errors.  A pair is
+    # rotated while it is above 1e-16 ||A||_F, so the mean square stays below that; V^H (A V) itself is
+    # evaluated to about 2 U ||A||_2, of the order of 2 U ||A||_F / sqrt(m) here (all eigenvalues near -1)
+    rng = np.random.default_rng(m)
+    A = rng.standard_normal((m, m)) + 1j * rng.standard_normal((m, m))
+    A = np.diag(-1.0 + 0.05 * rng.uniform(size=m)) + 0.5e-7 * (A + A.conj().T)
+    with cb.Solver(320, 320) as s:
+        V = cb.chfsi_heev(s.ctx, torch.from_numpy(A).cuda())[1].cpu().numpy()
+    left = V.conj().T @ (A @ V)
+    np.fill_diagonal(left, 0.0)
+    assert np.linalg.norm(left) / m <= (1e-16 + 2 * U / np.sqrt(m)) * np.linalg.norm(A)
