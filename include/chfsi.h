@@ -196,8 +196,8 @@ int chfsi_filter(chfsi_ctx* ctx, int64_t n, int32_t m, const chfsi_z* H, int64_t
 
 /* The same filter with split-BF16 tensor-core products (mixed-precision filter): every
  * product Hs*Y is computed from `slices` 7-bit digit slices of each FP64 operand (power-of-
- * two scales per row of H and per column of Y), exact in FP32 per 960-term chunk, combined
- * in double-float; relative error about 2^(-7 slices) of the operands' scales.
+ * two scales per row of H and per column of Y), exact in FP32 per chunk of 384 to 960
+ * terms, combined in double-float; relative error about 2^(-7 slices) of the operands' scales.
  * slices in [1, 8].  H must be Hermitian (full storage). */
 int chfsi_filter_split(chfsi_ctx* ctx, int64_t n, int32_t m, const chfsi_z* H, int64_t ldh,
                        chfsi_z* Y, int64_t ldy, const int32_t* degrees, double a0, double a,

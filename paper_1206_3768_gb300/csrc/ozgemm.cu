@@ -9,10 +9,10 @@
 //     Y^(k, j) = 2^{eB(j)} sum_t b_t(k, j) 2^{-7 t}
 //
 // with power-of-two scales per (complex) row of Hs and per column of Y.  Every digit is an
-// integer that bf16 holds exactly, every digit product is exact in FP32, and a sum of at
-// most 960 such products stays below 2^24, so each K-chunk of 960 accumulates EXACTLY in
-// the FP32 accumulators of mma.sync.m16n8k16 (bf16 inputs, FP32 accumulation).  Chunks
-// are scaled by 2^{-7(s+t)} (exact) and summed in double-float (FP32 pairs), and slice
+// integer that bf16 holds exactly, every digit product is exact in FP32, and a K-chunk short
+// enough that its sums stay below 2^24 accumulates EXACTLY in FP32 accumulators: 960 terms
+// where a slice pair has an accumulator to itself (the mma.sync kernel), 384 to 960, by S,
+// where the pairs of a level s + t share one (the tcgen05 kernel).  Chunks are scaled by 2^{-7(s+t)} (exact) and summed in double-float (FP32 pairs), and slice
 // pairs with s + t <= S + 1 are kept.  The truncation error of the kept pairs is about
 // 2^{-7S} relative to the row and column scales, so S = 7 gives FP64-level products and
 // S = 3 about 1e-6, at 6 ... 28 tensor-core GEMMs per product instead of FP64 FMAs (which
@@ -1224,10 +1224,6 @@ static bool oz_autotune() {
     return !(e && std::strcmp(e, "0") == 0);
   }();
   return v;
-}
-int oz_tuned_shapes() {
-  std::lock_guard<std::mutex> lk(g_tune_mu);
-  return (int)g_tune.size();
 }
 // Product kernel: tcgen05 (default) or the mma.sync kernel, chosen once per process by the
 // environment variable CHFSI_OZ_KERNEL ("tc" or "mma").
