@@ -30,6 +30,7 @@
 #include <utility>
 #include <vector>
 
+#include "digit_plan.cuh"
 #include "internal.cuh"
 
 namespace {
@@ -274,15 +275,22 @@ __global__ void oz_mma_epilogue_kernel(const double* part, int splits, int Mp, i
 // pairs (s, t) are issued from shared memory: 168 KB for 3584 clocks at S = 7, a third of the
 // bytes per flop.  Pairs of one level s + t carry the same scale 2^{-7 (s + t)} and add into
 // one accumulator, so S levels x 64 columns fit the 512 columns of tensor memory; the A slice s
-// meets the slices t = 1.. of B in ONE instruction of N = (number of levels) x w columns
-// (consecutive slices of B are consecutive rows of the stage, consecutive levels consecutive
-// accumulator columns), which also reads the A tile from shared memory once for several pairs.
+// meets several consecutive slices of B in ONE instruction of N = (levels of a group) x w
+// columns (consecutive slices of B are consecutive rows of the stage, consecutive levels
+// consecutive accumulator columns), which also reads the A tile from shared memory once for
+// several pairs.  The groups are fixed (digit_plan.cuh): all instructions that add into a column
+// have the same accumulator and shape, the condition under which they execute in issue order.
+// Where a slice reaches a part of a group only, the other levels meet the zeros in front of
+// slice 0 of B: at 7 slices 64 columns wide 31 slice products for 28, 4032 clocks a K-block.  (One
+// instruction over all levels that a slice reaches, 3712 clocks, would overlap accumulators of
+// different shapes, whose order nothing promises: filter of 20 steps at n = 9300, m = 320 58.6 ms,
+// 61.0 with groups.)
 // Exactness: |digit 1| <= 129 and the others <= 64, so level l adds at most 129^2 (l = 2) or
-// 2 129 64 + (l - 3) 64^2 per k; a chunk of tc_chunk_kb(S) K-blocks keeps every level below
+// 2 129 64 + (l - 3) 64^2 per k; a chunk of digit::chunk_blocks(S) K-blocks keeps every level below
 // 2^24 and each chunk is exact in the FP32 accumulators.  Sixteen drain warps then add the
 // levels into double-float sums (hi, lo) held in their registers.
-// Regions: levels are split into regions of at most 256 accumulator columns (columns 0 and
-// 256).  With one region (S w <= 256) chunks alternate between the two halves of tensor
+// Regions: groups of levels are split into regions of at most 256 accumulator columns (columns 0
+// and 256).  With one region (S w <= 256) chunks alternate between the two halves of tensor
 // memory; with two, the first and the last K-block of a chunk issue region 0 (the larger
 // products) and then region 1, so that draining region 0 overlaps the last products of region
 // 1, and draining region 1 the first products of region 0 of the next chunk.
@@ -296,8 +304,8 @@ __global__ void oz_mma_epilogue_kernel(const double* part, int splits, int Mp, i
 // runs out sets DEV_TIMEOUT and the CTA unwinds (waiting, again bounded, for its own copies
 // and MMAs) before freeing tensor memory.
 constexpr int TC_BM = 128, TC_BK = 64;
-constexpr int TC_W = 64;                                   // widest column tile
-constexpr int TC_REGION = 256;                             // accumulator columns of a region
+constexpr int TC_W = digit::WIDEST;                        // widest column tile
+constexpr int TC_REGION = digit::REGION;                   // accumulator columns of a region
 constexpr int TC_DWQ = 4;                                  // drain warps per 32-lane quarter
 constexpr int TC_THREADS = 64 + 32 * 4 * TC_DWQ;           // producer, MMA issuer, drain warps
 constexpr int TC_MAX_A = 12, TC_MAX_B = 4;                 // ring depths
@@ -309,25 +317,15 @@ constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;              // 16 KB per A tile
 // per term).  One instruction instead of seven per value.  From level 6 on it would cost
 // accuracy (reduction of n = 4096 with 8 slices: 3.4e-14 against 6.3e-15).
 constexpr int TC_LOW_LEVEL = 7;
-static_assert(8 * TC_W <= 512 && TC_W * (TC_REGION / TC_W) == TC_REGION && TC_W % 16 == 0 &&
-                  8 <= 2 * (TC_REGION / TC_W),
-              "eight levels fit two regions");
+static_assert(TC_BK == digit::BLOCK_K && TC_W % 16 == 0 && 8 * TC_W <= 2 * TC_REGION, "eight levels fit two regions");
 constexpr long kMbarSpinLimit = 1L << 26;
-
-// K-blocks of 64 per exact chunk: the largest count that keeps the largest level below 2^24.
-constexpr int tc_chunk_kb(int S) {
-  const int top = 2 * 129 * 64 + (S - 2) * 64 * 64;  // level S + 1 (S >= 2)
-  const int per_k = S >= 3 && top > 129 * 129 ? top : 129 * 129;
-  return (1 << 24) / (per_k * TC_BK);
-}
-static_assert(tc_chunk_kb(1) == 15 && tc_chunk_kb(2) == 15 && tc_chunk_kb(7) == 7 && tc_chunk_kb(8) == 6,
-              "exact chunks");
 
 struct TcParams {
   int a_lower, c_lower;                      // as in OzParams
   int b_tri;                                 // op(B) (complex) zero for k > j (1) or k < j (2)
   int S;                                     // slices (levels)
   int w;                                     // columns per tile (multiple of 16, <= TC_W)
+  int group, zeros, U;                       // levels of a group, zero slices of B, levels of region 0
   int nkb, tiles_m, tiles_n, raster, splits, Mp, Np;
   int na, nb;                                // ring depths: A tiles, B stages
   int chunk_kb;                              // K-blocks per exact chunk
@@ -440,7 +438,7 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 
 // The MMA issuer's state: one elected thread walks the K-blocks of its CTA.
 struct IssueArgs {
-  uint32_t sA, sB, b_slice, b_stage;               // shared-memory addresses and sizes
+  uint32_t sA, sB, b_slice, b_stage;               // shared-memory addresses (sB: slice 0) and sizes
   uint32_t fullA, emptyA, fullB, emptyB, accf, acce;  // mbarriers
   uint32_t tmem;
   int w, NA, NB, kb_lo, kb_hi, chunk_kb;
@@ -462,12 +460,13 @@ __device__ __forceinline__ uint64_t desc_from(uint32_t lo, uint32_t hi) {
   return d;
 }
 
-// S slices, U levels per region.  A K-block is S waits, up to 2 S groups of four products and S
-// commits; the loops over slices and regions are unrolled because one thread issues all of it
-// and its address arithmetic, not the tensor pipe, set the pace of a rolled loop (n = 9300, m =
-// 320: 3.5 ms a product).
-template <int S, int U>
+// S slices, levels in groups of G.  A K-block is S waits, a group of four products for every slice and
+// group of levels that it reaches, and S commits; the loops over slices and groups are unrolled
+// because one thread issues all of it and its address arithmetic, not the tensor pipe, set the
+// pace of a rolled loop (n = 9300, m = 320: 3.5 ms a product).
+template <int S, int G>
 __device__ __forceinline__ void issue_products(const IssueArgs& a) {
+  constexpr int U = digit::region_levels(S, G, digit::widest_with(G));  // levels of region 0
   constexpr int NREG = S > U ? 2 : 1;
   const uint32_t desc_hi = (uint32_t)(sw128_desc(0) >> 32), desc_lo = (uint32_t)sw128_desc(0);
   const uint32_t idesc0 = idesc_bf16(TC_BM, 0), idesc_w = (uint32_t)(a.w >> 3) << 17;
@@ -480,10 +479,9 @@ __device__ __forceinline__ void issue_products(const IssueArgs& a) {
       if (!issue_wait(a.fullB + 8 * sb, pb, a)) return;
       const uint32_t b_lo = desc_lo + ((a.sB + (uint32_t)sb * a.b_stage) >> 4);
       const bool first = kb == k0, last = kb == k1 - 1;
-      // group of four products of slice s into region `reg`: levels max(l0, s) .. l1 - 1
+      // products of slice s into the groups of region `reg` that it reaches (the first product of
+      // a chunk, s = 0, reaches every level of every group and overwrites it)
       auto group = [&](int s, int reg, uint32_t a_lo) -> bool {
-        const int l0 = reg * U, l1 = S < l0 + U ? S : l0 + U;
-        const int lb = l0 > s ? l0 : s;
         const uint32_t r = NREG == 2 ? (uint32_t)reg : (uint32_t)(chunk & 1);
         if (s == 0 && first) {
           // the region is free once the drain has finished its previous use
@@ -491,14 +489,18 @@ __device__ __forceinline__ void issue_products(const IssueArgs& a) {
           if (use >= 1 && !issue_wait(a.acce + 8 * r, (use - 1) & 1, a)) return false;
           tc_fence_after();
         }
-        const uint32_t idesc = idesc0 + (uint32_t)(l1 - lb) * idesc_w;
-        const uint32_t d = a.tmem + r * TC_REGION + (uint32_t)((lb - l0) * a.w);
-        const uint32_t bl = b_lo + (uint32_t)(lb - s) * b_slice16;
-        // the first product of a chunk (s = 0 reaches every level) overwrites the region
         const uint32_t keep = (s == 0 && first) ? 0u : 1u;
 #pragma unroll
-        for (int kk = 0; kk < TC_BK / 16; ++kk)  // 16 k = 32 bytes = 2 descriptor units
-          tc_mma(d, desc_from(a_lo + 2 * kk, desc_hi), desc_from(bl + 2 * kk, desc_hi), idesc, kk ? 1u : keep);
+        for (int i = 0; i < digit::groups(S, G); ++i) {
+          const digit::Product q = digit::product(S, G, U, s, i);
+          if (q.region != reg || q.levels == 0) continue;
+          const uint32_t idesc = idesc0 + (uint32_t)q.levels * idesc_w;
+          const uint32_t d = a.tmem + r * TC_REGION + (uint32_t)(q.at * a.w);
+          const uint32_t bl = b_lo + (uint32_t)q.first * b_slice16;
+#pragma unroll
+          for (int kk = 0; kk < TC_BK / 16; ++kk)  // 16 k = 32 bytes = 2 descriptor units
+            tc_mma(d, desc_from(a_lo + 2 * kk, desc_hi), desc_from(bl + 2 * kk, desc_hi), idesc, kk ? 1u : keep);
+        }
         return true;
       };
       int slot = sa;
@@ -566,7 +568,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const uintptr_t base = (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023;
   unsigned char* sA = reinterpret_cast<unsigned char*>(base);
   const int S = p.S, w = p.w, NA = p.na, NB = p.nb;
-  const uint32_t b_slice = (uint32_t)w * (TC_BK * 2), b_stage = (uint32_t)S * b_slice;  // multiples of 2048
+  // a B stage: the zero slices, then the S slices (all multiples of 2048 bytes)
+  const uint32_t b_slice = (uint32_t)w * (TC_BK * 2), b_zeros = (uint32_t)p.zeros * b_slice;
+  const uint32_t b_copy = (uint32_t)S * b_slice, b_stage = b_zeros + b_copy;
   unsigned char* sB = sA + NA * TC_A_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sB + NB * b_stage);
   // bars: fullA[NA], emptyA[NA], fullB[NB], emptyB[NB], accf[2], acce[2], done[1]
@@ -599,10 +603,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   const int per = (nkb - kb_first + p.splits - 1) / p.splits;
   const int kb_lo = min(nkb, kb_first + (int)blockIdx.y * per);
   const int kb_hi = min(nkb, kb_lo + per);
-  const int U = min(S, TC_REGION / w);  // levels per region
+  const int U = p.U;  // levels of region 0
   const int nreg = S > U ? 2 : 1;
 
-  const uint32_t sA_u = smem_u32(sA), sB_u = smem_u32(sB);
+  const uint32_t sA_u = smem_u32(sA), sB_u = smem_u32(sB) + b_zeros;  // slice 0 of the first stage
   const uint32_t fullA = smem_u32(bars), emptyA = fullA + 8 * NA;
   const uint32_t fullB = emptyA + 8 * NA, emptyB = fullB + 8 * NB;
   const uint32_t accf0 = emptyB + 8 * NB, acce0 = accf0 + 16, done_bar = acce0 + 16;
@@ -629,6 +633,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         smem_u32(tmem_slot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
+  for (uint32_t x = tid; x < NB * (b_zeros >> 4); x += TC_THREADS) {
+    const uint32_t stage = x / (b_zeros >> 4), at = x - stage * (b_zeros >> 4);
+    *reinterpret_cast<uint4*>(sB + stage * b_stage + 16 * at) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the tensor instructions read the zeros
   tc_fence_before();
   pdl_enter();  // set-up overlaps the end of the slicing; every thread waits before any copy or write
   __syncthreads();
@@ -645,7 +654,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       const int az = (int)blockIdx.z * p.a_zslices, bz = (int)blockIdx.z * p.b_zslices;
       for (int kb = kb_lo; kb < kb_hi && !stop; ++kb) {
         if (ib >= NB && !mbar_wait(emptyB + 8 * sb, pb ^ 1, abort_flag, p.status, p.spin_limit)) break;
-        mbar_expect_tx(fullB + 8 * sb, b_stage);
+        mbar_expect_tx(fullB + 8 * sb, b_copy);
         tma_load_3d(sB_u + (uint32_t)sb * b_stage, &tmB, kb * TC_BK, n0, bz, fullB + 8 * sb);
         ++ib;
         if (++sb == NB) {
@@ -689,24 +698,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       ia.tmem = tmem;
       ia.w = w; ia.NA = NA; ia.NB = NB; ia.kb_lo = kb_lo; ia.kb_hi = kb_hi; ia.chunk_kb = p.chunk_kb;
       ia.abort_flag = abort_flag; ia.status = p.status; ia.spin_limit = p.spin_limit;
-      // one unrolled loop per (slices, levels per region); U = 4 (w = 64) and 5 (w = 48) leave two
-      // regions for more slices than that, all other widths one
-      switch (nreg == 2 ? 16 * U + S : S) {
-        case 1: issue_products<1, 1>(ia); break;
-        case 2: issue_products<2, 2>(ia); break;
-        case 3: issue_products<3, 3>(ia); break;
-        case 4: issue_products<4, 4>(ia); break;
-        case 5: issue_products<5, 5>(ia); break;
-        case 6: issue_products<6, 6>(ia); break;
-        case 7: issue_products<7, 7>(ia); break;
-        case 8: issue_products<8, 8>(ia); break;
+      // one unrolled loop per (slices, levels of a group)
+      switch (16 * p.group + S) {
+        case 16 * 1 + 1: issue_products<1, 1>(ia); break;
+        case 16 * 2 + 2: issue_products<2, 2>(ia); break;
+        case 16 * 2 + 3: issue_products<3, 2>(ia); break;
+        case 16 * 3 + 3: issue_products<3, 3>(ia); break;
+        case 16 * 2 + 4: issue_products<4, 2>(ia); break;
+        case 16 * 3 + 4: issue_products<4, 3>(ia); break;
+        case 16 * 4 + 4: issue_products<4, 4>(ia); break;
+        case 16 * 2 + 5: issue_products<5, 2>(ia); break;
+        case 16 * 3 + 5: issue_products<5, 3>(ia); break;
         case 16 * 4 + 5: issue_products<5, 4>(ia); break;
+        case 16 * 2 + 6: issue_products<6, 2>(ia); break;
+        case 16 * 3 + 6: issue_products<6, 3>(ia); break;
         case 16 * 4 + 6: issue_products<6, 4>(ia); break;
+        case 16 * 2 + 7: issue_products<7, 2>(ia); break;
+        case 16 * 3 + 7: issue_products<7, 3>(ia); break;
         case 16 * 4 + 7: issue_products<7, 4>(ia); break;
+        case 16 * 2 + 8: issue_products<8, 2>(ia); break;
+        case 16 * 3 + 8: issue_products<8, 3>(ia); break;
         case 16 * 4 + 8: issue_products<8, 4>(ia); break;
-        case 16 * 5 + 6: issue_products<6, 5>(ia); break;
-        case 16 * 5 + 7: issue_products<7, 5>(ia); break;
-        case 16 * 5 + 8: issue_products<8, 5>(ia); break;
         default: break;  // no other (S, w) is launched
       }
       // all MMAs issued by this thread are complete once done_bar fires
@@ -734,7 +746,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         break;
       }
       tc_fence_after();
-      const int l0 = (nreg == 2 && r) ? U : 0, nl = min(S - l0, U);
+      const int l0 = (nreg == 2 && r) ? U : 0, nl = l0 ? S - U : U;  // the levels of this region
       const uint32_t acc_base = lane_base + (uint32_t)(r * TC_REGION);
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -1171,13 +1183,13 @@ int choose_oz_splits(int tiles, int total_kb, size_t cap_elems, int64_t tile_ele
 }
 
 // Split count for the tcgen05 kernel: split y takes k-blocks [y per, (y + 1) per) of every
-// tile.  Modelled time in clocks: a K-block costs its tensor work (2 w clocks per slice pair)
-// or its bytes at 36 per clock, a CTA about 5000 more (pipeline fill, last drain, partial
+// tile.  Modelled time in clocks: a K-block costs its tensor work (digit::block_clocks) or its
+// bytes at 36 per clock, a CTA about 5000 more (pipeline fill, last drain, partial
 // sums), and the launch is that times the waves of one CTA per SM; every split adds a write
 // and a read of the partial sums (16 bytes each, about 2800 bytes per clock over the GPU).
 int choose_tc_splits(int tiles, int nz, int nkb, int S, int w, size_t cap_elems, int64_t prod_elems) {
   const int sms = sm_count();
-  const double kb_cost = std::max(S * (S + 1) * (double)w, S * (TC_A_BYTES + 128.0 * w) / 36.0);
+  const double kb_cost = std::max((double)digit::block_clocks(S, w), S * (TC_A_BYTES + 128.0 * w) / 36.0);
   int best = 1;
   double best_cost = 1e300;
   for (int sp = 1; sp <= std::min(nkb, 64); ++sp) {
@@ -1427,7 +1439,7 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     tp.kfac = nz > 1 ? 1 : 2;
     tp.a_zslices = nz > 1 ? a.S : 0;
     tp.b_zslices = nz > 1 ? b.S : 0;
-    tp.chunk_kb = tc_chunk_kb(S);
+    tp.chunk_kb = digit::chunk_blocks(S);
     // first-level waits: the context's bound (a test hook) or the default; the waits that
     // let issued copies and MMAs finish after an abort always use the default
     tp.spin_limit = oz.wait_limit > 0 ? oz.wait_limit : kMbarSpinLimit;
@@ -1439,15 +1451,17 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     // one time (152) cover about 10 row tiles x 16 column tiles of a wide product
     tp.raster = std::min(tp.tiles_n, 16);
     const int tiles = tp.tiles_m * tp.tiles_n;
-    const int b_stage = S * tp.w * TC_BK * 2;
+    tp.group = digit::group_levels(S, tp.w);
+    tp.zeros = digit::zero_slices(tp.group);
+    tp.U = digit::region_levels(S, tp.group, tp.w);
+    const int b_stage = (S + tp.zeros) * tp.w * TC_BK * 2;
     // rings: two B stages (more while a B stage is small against the A tiles of a K-block), the
     // rest of the shared memory for A tiles (at least the slices of region 0 stay resident)
     tp.nb = 2;
     while (tp.nb < TC_MAX_B && (tp.nb + 1) * b_stage + std::min(2 * S, TC_MAX_A) * TC_A_BYTES <= TC_SMEM_BUDGET)
       ++tp.nb;
     tp.na = std::min(TC_MAX_A, (TC_SMEM_BUDGET - tp.nb * b_stage) / TC_A_BYTES);
-    const int levels_per_region = TC_REGION / tp.w;
-    if (tp.na < (S > levels_per_region ? levels_per_region + 1 : 2)) return cudaErrorInvalidValue;
+    if (tp.na < (S > tp.U ? tp.U + 1 : 2)) return cudaErrorInvalidValue;
     CUtensorMap mapA, mapB;
     const int kr = nz > 1 ? a.K : 2 * a.K;  // real k extent of both operands
     if (!encode_bf16_map(&mapA, a.ptr, kr, Kp, nz > 1 ? a.M : 2 * a.M, a.slice, nz * a.S, TC_BM, 1) ||
