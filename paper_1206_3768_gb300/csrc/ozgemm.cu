@@ -288,7 +288,9 @@ __global__ void oz_mma_epilogue_kernel(const double* part, int splits, int Mp, i
 // Exactness: |digit 1| <= 129 and the others <= 64, so level l adds at most 129^2 (l = 2) or
 // 2 129 64 + (l - 3) 64^2 per k; a chunk of digit::chunk_blocks(S) K-blocks keeps every level below
 // 2^24 and each chunk is exact in the FP32 accumulators.  Sixteen drain warps then add the
-// levels into double-float sums (hi, lo) held in their registers.
+// levels into double-float sums (hi, lo) held in their registers, every level by two-sum: levels
+// s + t >= 7 in the low word alone would lose what passes its 24 bits (sums of one level above
+// 2^24; filter of 20 steps at n = 9300, m = 320 61.6 ms, 63.1 with two-sum for all).
 // Regions: groups of levels are split into regions of at most 256 accumulator columns (columns 0
 // and 256).  With one region (S w <= 256) chunks alternate between the two halves of tensor
 // memory; with two, the first and the last K-block of a chunk issue region 0 (the larger
@@ -311,12 +313,6 @@ constexpr int TC_THREADS = 64 + 32 * 4 * TC_DWQ;           // producer, MMA issu
 constexpr int TC_MAX_A = 12, TC_MAX_B = 4;                 // ring depths
 constexpr int TC_SMEM_BUDGET = 227 * 1024 - 1024 - 512;    // dynamic shared memory for the rings
 constexpr int TC_A_BYTES = TC_BM * TC_BK * 2;              // 16 KB per A tile
-// Levels from this one on (s + t >= 7) go straight into the low word: a chunk of level 7 is about
-// 2^-33 of the operands' scales, so its rounding there is 2^-24 of that, below the rounding of
-// the low word itself (2^-48 of a sum near the scales) and the dropped pairs of 8 slices (2^-58
-// per term).  One instruction instead of seven per value.  From level 6 on it would cost
-// accuracy (reduction of n = 4096 with 8 slices: 3.4e-14 against 6.3e-15).
-constexpr int TC_LOW_LEVEL = 7;
 static_assert(TC_BK == digit::BLOCK_K && TC_W % 16 == 0 && 8 * TC_W <= 2 * TC_REGION, "eight levels fit two regions");
 constexpr long kMbarSpinLimit = 1L << 26;
 
@@ -762,15 +758,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int q = 0; q < 4; ++q)
               if (l + q < nl) {
                 // level l0 + l + q (0-based) carries 2^{-7 (level + 2)}
-                const int level = l0 + l + q + 2;
-                const float sc = __int_as_float((127 - OZ_BETA * level) << 23);
-                if (level < TC_LOW_LEVEL) {
+                const float sc = __int_as_float((127 - OZ_BETA * (l0 + l + q + 2)) << 23);
 #pragma unroll
-                  for (int c = 0; c < 8; ++c) two_sum_scaled(hi[i][c], lo[i][c], __uint_as_float(acc[q][c]), sc);
-                } else {
-#pragma unroll
-                  for (int c = 0; c < 8; ++c) lo[i][c] = fmaf(__uint_as_float(acc[q][c]), sc, lo[i][c]);
-                }
+                for (int c = 0; c < 8; ++c) two_sum_scaled(hi[i][c], lo[i][c], __uint_as_float(acc[q][c]), sc);
               }
           }
         }
