@@ -1198,13 +1198,14 @@ int choose_tc_splits(int tiles, int nz, int nkb, int S, int w, size_t cap_elems,
 // ---------------------------------------------------------------------------- host side
 // Autotuner of the tcgen05 kernel's split count: the best configuration measured for each
 // product shape, shared by all contexts of the process (batch workers tune from several host
-// threads).  Environment variable CHFSI_OZ_AUTOTUNE=0 keeps the wave model's choice.
+// threads) whose partial sums allow the same counts: max_splits, the most that a context could
+// choose, is part of the key, so that no count is larger than the context has room for.  Environment variable CHFSI_OZ_AUTOTUNE=0 keeps the wave model's choice.
 struct TuneKey {
-  int Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz;
+  int Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz, max_splits;
   bool operator<(const TuneKey& o) const {
-    const int a[9] = {Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz};
-    const int b[9] = {o.Mp, o.Np, o.Kp, o.S, o.a_lower, o.c_lower, o.w, o.b_tri, o.nz};
-    return std::lexicographical_compare(a, a + 9, b, b + 9);
+    const int a[10] = {Mp, Np, Kp, S, a_lower, c_lower, w, b_tri, nz, max_splits};
+    const int b[10] = {o.Mp, o.Np, o.Kp, o.S, o.a_lower, o.c_lower, o.w, o.b_tri, o.nz, o.max_splits};
+    return std::lexicographical_compare(a, a + 10, b, b + 10);
   }
 };
 static std::mutex g_tune_mu;
@@ -1402,7 +1403,7 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
   if (S > b.S || S > a.S || S < 1 || a.Kp != b.Kp || a.nz != b.nz) return cudaErrorInvalidValue;
   const int nz = a.nz;  // 3: Gauss form (tcgen05 path only)
   if (nz != 1 && (nz != 3 || !oz_use_tcgen05())) return cudaErrorInvalidValue;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   // Pairs (s, t) with s + t <= S + 1, grouped by the A slice s so that consecutive pairs
   // stream the same slice of the large operand (it stays in L2 between them).
   OzPairs pairs;
@@ -1471,14 +1472,15 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
     const size_t part_cap = oz.part_elems / (size_t)nz;  // partials of each of the nz products
     const int model_splits = choose_tc_splits(tiles, nz, tp.nkb, S, tp.w, part_cap, (int64_t)Mp * Np);
     splits = model_splits;
-    const TuneKey key{Mp, Np, Kp, S, a_lower, c_lower, tp.w, b_tri, nz};
+    const int max_splits = (int)std::min<size_t>(std::min(tp.nkb, 64), part_cap / ((size_t)Mp * Np));
+    if (max_splits < 1) return cudaErrorInvalidValue;
+    const TuneKey key{Mp, Np, Kp, S, a_lower, c_lower, tp.w, b_tri, nz, max_splits};
     if (oz_autotune() && !tune_lookup(key, &splits)) {
       cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         std::vector<int> cand;
         for (int num : {2, 3, 4, 6, 8}) {  // model x {1/2, 3/4, 1, 3/2, 2}
-          const int sp = std::max(1, std::min(std::min(tp.nkb, 64), (model_splits * num + 2) / 4));
-          if ((size_t)sp * (size_t)((int64_t)Mp * Np) > part_cap) continue;
+          const int sp = std::max(1, std::min(max_splits, (model_splits * num + 2) / 4));
           if (std::find(cand.begin(), cand.end(), sp) == cand.end()) cand.push_back(sp);
         }
         cudaEvent_t t0, t1;
@@ -1501,7 +1503,6 @@ cudaError_t oz_product(const OzA& a, const OzB& b, int S, double alpha, double b
         tune_store(key, splits);
       }
     }
-    if ((size_t)splits * (size_t)nz * (size_t)Mp * (size_t)Np > oz.part_elems) return cudaErrorInvalidValue;
     if (ev_gemm_begin) cudaEventRecord(ev_gemm_begin, s);
     e = launch(splits);
     if (ev_gemm_end) cudaEventRecord(ev_gemm_end, s);
