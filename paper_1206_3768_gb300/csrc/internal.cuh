@@ -202,8 +202,8 @@ cudaError_t lanczos_next(const zd* w, int n, const double* norm2, const zd* c, i
                          double* beta, zd* dst, cudaStream_t s);
 cudaError_t vec_norm(const zd* w, int n, double* out, cudaStream_t s);
 cudaError_t vec_scale_into(const zd* w, int n, const double* nrm, zd* dst, cudaStream_t s);
-cudaError_t tridiag_extremes(const double* alpha, const double* beta, int k, double* out3,
-                             cudaStream_t s);
+// Extreme eigenvalues of T_k (alpha and beta may be scaled in place) and the largest + |beta_{k-1}|.
+cudaError_t tridiag_extremes(double* alpha, double* beta, int k, double* out3, cudaStream_t s);
 
 // ------------------------------------------------------------------ split-BF16 products
 struct OzA {                        // A operand: S digit slices of op(A) (M x K complex)

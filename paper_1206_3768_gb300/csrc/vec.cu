@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(HEMV_THREADS)
 // clocks an instruction of a warp) and how many SMs take part, so each dot product is shared by
 // DOT_PARTS CTAs, a row of the update by four lanes, and the pieces (few and in a fixed order) are
 // added where they are read.
-constexpr int DOT_PARTS = 4, UPD_ROWS = 64;
+constexpr int DOT_PARTS = 4, UPD_ROWS = 64, UPD_COEFS = 1024;  // coefficients in shared memory at a time
 
 // c[l * DOT_PARTS + q] = part q of V_l^H w, l = 0..j.  Grid: (j + 1, DOT_PARTS).
 __global__ void block_dots_kernel(const zd* V, int64_t ldv, const zd* w, int n, zd* c) {
@@ -607,14 +607,19 @@ __device__ __forceinline__ zd dot_total(const zd* c, int l) {
 // w -= V c; norm2 (optional): sum of |w_i|^2 over the CTA's rows.  UPD_ROWS rows a CTA, four lanes each.
 __global__ void __launch_bounds__(4 * UPD_ROWS)
     block_update_kernel(const zd* V, int64_t ldv, int jp1, const zd* c, zd* w, int n, double* norm2) {
-  extern __shared__ zd cs[];
-  for (int l = threadIdx.x; l < jp1; l += blockDim.x) cs[l] = dot_total(c, l);
-  __syncthreads();
+  __shared__ zd cs[UPD_COEFS];
   const int i = blockIdx.x * UPD_ROWS + (threadIdx.x >> 2), q = threadIdx.x & 3;
   zd s = zmk(0.0, 0.0);
-  if (i < n) {
+  for (int l0 = 0; l0 < jp1; l0 += UPD_COEFS) {
+    const int cnt = min(UPD_COEFS, jp1 - l0);
+    if (l0) __syncthreads();  // the coefficients before have been used
+    for (int l = threadIdx.x; l < cnt; l += blockDim.x) cs[l] = dot_total(c, l0 + l);
+    __syncthreads();
+    if (i < n) {
+      const zd* v = V + i + (int64_t)l0 * ldv;
 #pragma unroll 4
-    for (int l = q; l < jp1; l += 4) s = zfma(V[i + (int64_t)l * ldv], cs[l], s);
+      for (int l = q; l < cnt; l += 4) s = zfma(v[(int64_t)l * ldv], cs[l], s);
+    }
   }
 #pragma unroll
   for (int o = 1; o < 4; o <<= 1) {
@@ -694,10 +699,15 @@ __device__ int sturm_count(const double* al, const double* b2, int k, double x) 
 // out[0] = min eig(T_k), out[1] = max eig(T_k), out[2] = max eig + |beta_{k-1}|: warp 0 looks for the
 // smallest, warp 1 for the largest eigenvalue, 32 points of the interval at a time (an interval
 // shrinks by 33 a round, to neighbouring doubles in about 11; one thread bisecting with divisions
-// took 1.1 ms at k = 20 and 2.2 ms at k = 40).  T is scaled by a power of two to a bound in [1/2, 1).
-__global__ void __launch_bounds__(64) tridiag_extremes_kernel(const double* al, const double* be, int k, double* out) {
-  extern __shared__ double tri[];  // k: scaled diagonal; k: scaled squared off-diagonal
+// took 1.1 ms at k = 20 and 2.2 ms at k = 40).  T is scaled by a power of two to a bound in [1/2, 1),
+// in shared memory up to TRIDIAG_SMEM rows, else where it is.
+constexpr int TRIDIAG_SMEM = 2048;
+__global__ void __launch_bounds__(64) tridiag_extremes_kernel(double* al, double* be, int k, double* out) {
+  __shared__ double sal[TRIDIAG_SMEM], sb2[TRIDIAG_SMEM];
   __shared__ double ext[2];
+  double* sa = k <= TRIDIAG_SMEM ? sal : al;  // scaled diagonal
+  double* sb = k <= TRIDIAG_SMEM ? sb2 : be;  // scaled squared off-diagonal
+  const double last = fabs(be[k - 1]);
   const int tid = threadIdx.x, lane = tid & 31;
   double lo = INFINITY, hi = -INFINITY;
   for (int i = lane; i < k; i += 32) {
@@ -714,10 +724,11 @@ __global__ void __launch_bounds__(64) tridiag_extremes_kernel(const double* al, 
   const double bound = fmax(fabs(lo), fabs(hi));
   if (bound > 0.0 && isfinite(bound)) frexp(bound, &shift);
   const double down = ldexp(1.0, -shift);
+  __syncthreads();  // both warps have read T
   for (int i = tid; i < k; i += 64) {
     const double b = i < k - 1 ? be[i] * down : 0.0;
-    tri[i] = al[i] * down;
-    tri[k + i] = b * b;
+    sa[i] = al[i] * down;
+    sb[i] = b * b;
   }
   lo *= down;
   hi *= down;
@@ -729,7 +740,7 @@ __global__ void __launch_bounds__(64) tridiag_extremes_kernel(const double* al, 
   for (int round = 0; round < 40 && b > a; ++round) {
     const double x = fma((b - a) * (1.0 / 33.0), (double)(lane + 1), a);
     const bool inside = x > a && x < b;
-    const unsigned at = __ballot_sync(0xffffffffu, inside && sturm_count(tri, tri + k, k, x) >= want);
+    const unsigned at = __ballot_sync(0xffffffffu, inside && sturm_count(sa, sb, k, x) >= want);
     const unsigned in = __ballot_sync(0xffffffffu, inside);
     if (in == 0u) break;  // no double between a and b
     const unsigned below = in & ~at;  // points inside that do not reach it
@@ -747,7 +758,7 @@ __global__ void __launch_bounds__(64) tridiag_extremes_kernel(const double* al, 
   if (tid == 0) {
     out[0] = ext[0];
     out[1] = ext[1];
-    out[2] = ext[1] + fabs(be[k - 1]);
+    out[2] = ext[1] + last;
   }
 }
 
@@ -1061,13 +1072,7 @@ cudaError_t block_dots(const zd* V, int64_t ldv, int j, const zd* w, int n, zd* 
   return cudaGetLastError();
 }
 cudaError_t block_update(const zd* V, int64_t ldv, int j, const zd* c, zd* w, int n, double* norm2, cudaStream_t s) {
-  const size_t smem = sizeof(zd) * (size_t)(j + 1);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(block_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  block_update_kernel<<<(n + UPD_ROWS - 1) / UPD_ROWS, 4 * UPD_ROWS, smem, s>>>(V, ldv, j + 1, c, w, n, norm2);
+  block_update_kernel<<<(n + UPD_ROWS - 1) / UPD_ROWS, 4 * UPD_ROWS, 0, s>>>(V, ldv, j + 1, c, w, n, norm2);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
@@ -1088,15 +1093,8 @@ cudaError_t vec_scale_into(const zd* w, int n, const double* nrm, zd* dst, cudaS
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
-cudaError_t tridiag_extremes(const double* alpha, const double* beta, int k, double* out3,
-                             cudaStream_t s) {
-  const size_t smem = 2 * sizeof(double) * (size_t)k;
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(tridiag_extremes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  tridiag_extremes_kernel<<<1, 64, smem, s>>>(alpha, beta, k, out3);
+cudaError_t tridiag_extremes(double* alpha, double* beta, int k, double* out3, cudaStream_t s) {
+  tridiag_extremes_kernel<<<1, 64, 0, s>>>(alpha, beta, k, out3);
   CHFSI_COUNT_LAUNCH();
   return cudaGetLastError();
 }
