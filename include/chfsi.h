@@ -250,7 +250,8 @@ int chfsi_degrees(chfsi_ctx* ctx, int32_t m, const double* theta, const double* 
 
 /* Eigen-decomposition of the m x m Hermitian matrix G (full storage, device): ascending
  * eigenvalues w (device) and orthonormal eigenvectors V (device, ld ldv), by cyclic
- * parallel Jacobi.  G is not modified. */
+ * parallel Jacobi.  G is not modified; its entries may lie anywhere in the range of FP64 (they
+ * are scaled by a power of two).  A G with a NaN or an infinity has NaN for every result. */
 int chfsi_heev(chfsi_ctx* ctx, int32_t m, const chfsi_z* G, int64_t ldg, double* w,
                chfsi_z* V, int64_t ldv);
 
