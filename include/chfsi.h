@@ -294,7 +294,11 @@ int chfsi_heev_noalloc(int32_t m, const chfsi_z* G, int64_t ldg, double* w, chfs
  * the kernel unwinds (letting its own copies and tensor-core operations finish first) and
  * returns, and the call reports CHFSI_ETIMEOUT with the context still usable.  0 (the
  * default) means a few seconds of polling, far above any normal wait; a small bound makes
- * the waits run out, which is how the timeout path is exercised.  Errors: EINVAL. */
+ * the waits run out, which is how the timeout path is exercised.  The hardware's barrier of
+ * a thread-block cluster is no such wait and has no limit: the CTAs of a cluster are resident
+ * together and all reach each barrier or all leave before it.  Two kernels use it, the panel
+ * factorisation of B and, while no bound is set here, the eigensolver on up to 64 columns
+ * (with a bound set every size runs over the grid barrier).  Errors: EINVAL. */
 int chfsi_set_wait_limit(chfsi_ctx* ctx, int64_t polls);
 
 /* Complex FP64 GEMM used by every dense step, exposed for testing:
