@@ -229,8 +229,8 @@ GemmDesc gd(int M, int N, int K, const zd* A, int64_t lda, int opA, const zd* B,
   return g;
 }
 
-// Panel width of the blocked factorisations (measured: 256-column panels made the n = 9300
-// workload's reduction phase slower, 2.90 s against 2.81 s per 20-problem step).
+// Panel width of the blocked factorisations: what the panel kernel takes (PC_MAX) and the rows that
+// one launch inverts per diagonal block.
 constexpr int NB = 128;
 // Outer panel of the Cholesky factorisation.
 constexpr int NB2 = 512;
@@ -373,7 +373,7 @@ int reduce_to_standard(chfsi_ctx* ctx, const zd* Af, int64_t lda, const zd* Linv
 int lanczos_issue(chfsi_ctx* ctx, cudaStream_t st, const zd* H, int64_t ldh, int n, int k, const zd* v0,
                   uint64_t seed, double* out3);
 
-// The launch-bound Lanczos loop (seven small kernels per step) is captured once per
+// The launch-bound Lanczos loop (six short kernels per step) is captured once per
 // (matrix, size, steps, seed, precision) on a private stream and replayed as a CUDA graph on
 // the context's stream; a caller start vector v0, or a failed capture, issues it directly.
 int lanczos_run(chfsi_ctx* ctx, const zd* H, int64_t ldh, int n, int k, const zd* v0,

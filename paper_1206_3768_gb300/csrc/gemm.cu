@@ -208,10 +208,12 @@ int sm_count() {
 // sequence (at most 30 columns) 66 -> 12 and 56 -> 11 us (one tile split 16 ways reached 16 SMs),
 // filter step n = 1024, m = 64 408 -> 365 us (608 CTAs of 4 unequal k-tiles before), 128 x 128 x 128
 // 103 -> 28 us.
-// A sum is split at least every CHAIN to 2 CHAIN terms where the partials have room: the rounding of
-// a serial sum grows with the root of its length, and up to n = 1300 a filter step with the splits
-// that balance alone would choose was up to 1.3 times further from the exact one than with the
-// former tile's many splits (with these 0.92 to 1.04 times, at the same speed within 1 %).
+// A sum is split at least every CHAIN to 2 CHAIN terms where that takes at most 64 splits and the
+// partials have room (above K = 8192 the pieces are K / 64 long; a triangular operand counts half
+// its K, so its longest sums are in pieces twice as long): the rounding of a serial sum grows with
+// the root of its length, and up to n = 1300 a filter step with the splits that balance alone would
+// choose was up to 1.3 times further from the exact one than with the former tile's many splits
+// (with these 0.92 to 1.04 times, at the same speed within 1 %).
 constexpr int CHAIN = 64;
 struct Shape {
   int R, splits, tiles_m, tiles_n;

@@ -297,9 +297,9 @@ __global__ void oz_mma_epilogue_kernel(const double* part, int splits, int Mp, i
 // products) and then region 1, so that draining region 0 overlaps the last products of region
 // 1, and draining region 1 the first products of region 0 of the next chunk.
 // Measured against the one-pair-per-stage kernel (Gauss form, 7 slices, one product): n = 9300,
-// m = 320 6.1 -> 2.6 ms, 1.76 PFLOP/s of slice-pair flops at the card's power cap (2010 to 2070
-// MHz, 1360 W); n = 5957, m = 37 0.82 -> 0.25 ms; with 5 slices n = 2600, m = 130 and fewer
-// columns 0.15 -> 0.07 ms.
+// m = 320 6.1 -> 2.85 ms, 1.63 PFLOP/s of slice-pair flops (at the card's power cap: SM clock 2010
+// to 2070 MHz); n = 5957, m = 37 0.82 -> 0.26 ms; with 5 slices n = 2600, m = 130 and fewer columns
+// 0.15 -> 0.07 ms.
 // Warp 0 issues TMA loads (a ring of A tiles and a ring of B stages), warp 1 issues MMAs, warps
 // 2..17 drain: four warps per group of 32 tensor-memory lanes, warp h of a group owns the
 // 8-column blocks h and h + 4 of the tile.  Every wait on an mbarrier is bounded; a wait that
